@@ -961,6 +961,7 @@ static skf_status build_layout(skf_csr *A, int cut, int sort, cudaStream_t st) {
         A->max_chunk_entries = std::max<int64_t>(A->max_chunk_entries, hoff[t1] - hoff[t0]);
     }
     const int64_t padded = hoff[A->nslices];
+    A->sell_entries = padded;
     if (cudaMalloc(&A->sell_val, esz * std::max<int64_t>(padded, 1)) != cudaSuccess ||
         cudaMalloc(&A->sell_col, sizeof(int32_t) * std::max<int64_t>(padded, 1)) != cudaSuccess) {
         cudaGetLastError();

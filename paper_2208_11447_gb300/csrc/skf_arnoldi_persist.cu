@@ -53,6 +53,10 @@ namespace {
 
 constexpr int kPT = 512;                      // threads per CTA
 constexpr int kPNW = kPT / 32;                // warps per CTA
+// rows per CTA below which CTAs are left out: 10^4 rows 12.4 / 9.6 / 9.6 us
+// per step at 512 / 256 / 128 rows, 25600 rows 13.7 / 10.6 / 10.9 us
+constexpr int kPersistMinRows = 256;
+constexpr int kFlushAll = 64;                 // slices per CTA up to which all warps add up the sketch bins
 constexpr long long kBarrierBudget = 1ll << 31;   // SM cycles (about one second)
 
 struct PCtx {
@@ -62,6 +66,7 @@ struct PCtx {
     const int32_t *sell_w;
     const void *sell_val;      // T values (T = double, or float for an FP32 basis)
     const int32_t *sell_col;
+    float l2_frac;             // share of the operator's lines kept in L2 from step to step
     SparseSign sp;
     const uint16_t *pattern;   // [n][zeta]
     const uint8_t *pattern8;   // [n][8] or nullptr
@@ -74,8 +79,10 @@ struct PCtx {
     int64_t ldv;
     double *vscale, *SV, *SAV, *H;
     int *iscal;
-    double *pA;                // [KW + 1][G]: window dots, max|y~|
-    double *pB;                // [KW + 1][G]: ||w||^2, max|w|, Gram entries
+    double *pB;                // [2][G]: partial ||b||^2, max|b|
+    unsigned long long *slot;  // [2 m + 1][kSlot]: exact sums of the window dots and max|y~| of step j at
+                               // 2 j, of ||w_j||^2, the Gram entries and max|w_j| at 2 j - 1 (see push_sums)
+    int e_row;                 // |(A x)_r| < 2^e_row max|x|
     unsigned long long *accw;  // [m][2][s]: limb sums of S w_j
     unsigned long long *accy;  // [2][s]: limb sums of the directly sketched y~
     double *Sw;                // s x m: S w_j (unnormalised)
@@ -95,29 +102,63 @@ __device__ __forceinline__ int ld_volatile_i32(const int *p) {
     return *(const volatile int *)p;
 }
 
+// Operator loads.  A is read once per step by the same CTA, so what decides is
+// whether it stays in L2 (129 MB) from one step to the next: `pol` keeps the
+// fraction l2_frac of its lines (evict_last) and streams the rest
+// (evict_first), so that an operator beyond the budget still finds that
+// fraction there instead of evicting itself.
+__device__ __forceinline__ unsigned long long operator_policy(float frac) {
+    unsigned long long p;
+    asm("createpolicy.fractional.L2::evict_last.L2::evict_first.b64 %0, %1;" : "=l"(p) : "f"(frac));
+    return p;
+}
+__device__ __forceinline__ double ld_op(const double *a, unsigned long long pol) {
+    double v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(a), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float ld_op(const float *a, unsigned long long pol) {
+    float v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ int ld_op(const int32_t *a, unsigned long long pol) {
+    int v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(a), "l"(pol));
+    return v;
+}
+
+// Wait (one thread) until *cnt reaches target; 0 if the wait ran out of budget
+// or another CTA's did, and then *flag is set.
+__device__ __forceinline__ int spin_until(const unsigned *cnt, unsigned target, int *flag, long long budget) {
+    const long long t0 = clock64();
+    while (ld_acquire_u32(cnt) < target) {
+        if (ld_volatile_i32(flag) != 0 || clock64() - t0 > budget) {
+            atomicExch(flag, 1);
+            return 0;
+        }
+    }
+    return 1;
+}
+
 // Grid-wide barrier number `nb` (1, 2, ...) of a co-resident grid: arrive,
 // then wait until nb * gridDim.x arrivals are visible.  Returns false (in
 // every thread of the CTA) if the wait ran out of budget or another CTA's
-// did; the first CTA to give up sets *flag.
+// did; the first CTA to give up sets *flag.  The arrival is a release and the
+// poll an acquire at GPU scope, and the block barriers on both sides extend
+// them to the whole CTA (cumulativity), so no further fence is needed; a
+// __threadfence() on each side cost 0.3 us per barrier (1.34 -> 1.12 us with
+// 10 CTAs, 2.45 -> 2.14 us with 152) and made the reduction before it wait
+// for the service warp's sketch atomics (5.5 -> 3.5 us at s = 960).
+__device__ __forceinline__ void grid_arrive(unsigned *bar) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+}
 __device__ bool grid_barrier(unsigned *bar, int *flag, unsigned nb, long long budget) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
-        const unsigned target = nb * gridDim.x;
-        const long long t0 = clock64();
-        int good = 1;
-        while (ld_acquire_u32(bar) < target) {
-            if (ld_volatile_i32(flag) != 0 || clock64() - t0 > budget) {
-                good = 0;
-                break;
-            }
-            // spin: one thread per CTA polls one L2 line
-        }
-        if (!good) atomicExch(flag, 1);
-        __threadfence();
-        ok = good;
+        grid_arrive(bar);
+        ok = spin_until(bar, nb * gridDim.x, flag, budget);   // one thread per CTA polls one L2 line
     }
     __syncthreads();
     return ok != 0;
@@ -200,17 +241,160 @@ __device__ __forceinline__ unsigned long long block_reduce_t0(double (&v)[NV], u
     return key;
 }
 
+// Grid-wide sums without floating-point additions.  The per-thread partials of
+// a phase (window dots; ||w||^2 and Gram entries) are cut into kCh chunks of
+// 22 bits of a 154-bit field below an exponent bound that every CTA knows, and
+// the chunks are added as integers: a warp reduction per chunk, a shared
+// atomic per warp, one 64-bit global atomic per CTA and chunk, issued just
+// before the CTA's barrier arrival.  Integer sums do not depend on the order,
+// so after the barrier one 7-word load replaces the read and fixed-order sum
+// of G partials, and no FP64 addition (65 dependent cycles each on this part,
+// 16 more of the SM's FP64 pipe) is left on the path from the last row to the
+// coefficients.  The sums are exact to 2^-154 of the bound.  Measured per step
+// from the last row to the coefficients: 7.3 -> 5.9 us (100^3 grid, 152 CTAs),
+// 7.0 -> 4.2 us (10^4 rows; 10 -> 40 CTAs).
+constexpr int kCh = 7, kChBits = 22;         // chunks of a sum
+constexpr int kField = kCh * kChBits;        // bits below the bound
+constexpr int kSlot = 32;                    // words of a slot: kCh per sum (at most 4), [30] not finite, [31] max key
+
+// x as signed chunks of x / 2^(E - kField); false if x is not finite or not
+// below 2^E in magnitude.
+__device__ __forceinline__ bool chunks_of(double x, int E, int (&ch)[kCh]) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    const int be = (int)((bits >> 52) & 0x7FFull);
+    const unsigned long long mant = be ? ((bits & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) : 0ull;
+    const int p = be - 1075 - (E - kField);   // position of the mantissa's lowest bit in the field
+    const bool ok = be != 0x7FF && (be == 0 || p <= kField - 53);
+    const bool neg = (bits >> 63) != 0ull;
+#pragma unroll
+    for (int i = 0; i < kCh; ++i) {
+        const int sh = kChBits * i - p;
+        unsigned long long v;
+        asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(mant), "r"(max(sh, 0)));   // shifts of 64 and more give 0
+        asm("shl.b64 %0, %1, %2;" : "=l"(v) : "l"(v), "r"(max(-sh, 0)));
+        const int d = (int)((unsigned)v & ((1u << kChBits) - 1u));
+        ch[i] = ok ? (neg ? -d : d) : 0;
+    }
+    return ok;
+}
+__device__ __forceinline__ bool chunks_of(float x, int E, int (&ch)[kCh]) {
+    const unsigned bits = __float_as_uint(x);
+    const int be = (int)((bits >> 23) & 0xFFu);
+    const unsigned mant = be ? ((bits & 0x7FFFFFu) | 0x800000u) : 0u;
+    const int p = be - 150 - (E - kField);
+    const bool ok = be != 0xFF && (be == 0 || p <= kField - 24);
+    const bool neg = (bits >> 31) != 0u;
+#pragma unroll
+    for (int i = 0; i < kCh; ++i) {
+        const int sh = kChBits * i - p;
+        unsigned v;
+        asm("shr.u32 %0, %1, %2;" : "=r"(v) : "r"(mant), "r"(max(sh, 0)));
+        asm("shl.b32 %0, %1, %2;" : "=r"(v) : "r"(v), "r"(max(-sh, 0)));
+        const int d = (int)(v & ((1u << kChBits) - 1u));
+        ch[i] = ok ? (neg ? -d : d) : 0;
+    }
+    return ok;
+}
+
+// Magnitudes as ordered 32-bit keys (the high word of a double), and the
+// exponent bound |x| < 2^E of the largest: only its exponent is needed.
+__device__ __forceinline__ unsigned mag_key(double x) {
+    return (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7FFFFFFFu;
+}
+__device__ __forceinline__ unsigned mag_key(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+template <typename T>
+__device__ __forceinline__ int key_exponent(unsigned key) {
+    constexpr bool F32 = sizeof(T) == 4;
+    const int be = (int)(key >> (F32 ? 23 : 20));
+    if (key == 0u || be == (F32 ? 0xFF : 0x7FF)) return kNoExp;   // zero (or below 2^-1042), or not finite
+    return max(be, 1) - (F32 ? 126 : 1022);
+}
+// E with |x| < 2^E (x finite)
+__device__ __forceinline__ int exponent_above(double x) {
+    return (int)(mag_key(x) >> 20) - 1022;
+}
+
+// Adds the first nv of the per-thread values v[] (|v[i]| < 2^E[i]) and the
+// maximum of the keys to this CTA's share of `slot`: warp reductions, shared
+// atomics, then one global atomic per chunk from warp 0, whose lane 0 may
+// arrive at the barrier after a __syncwarp().  sch: kSlot ints, zero on entry
+// and left zero.
+template <int KW, typename T>
+__device__ __forceinline__ void push_sums(const T (&v)[KW], int nv, const int *E, unsigned key, int *sch,
+                                          unsigned long long *slot) {
+    const int lane = threadIdx.x & 31;
+    int mine = 0;
+    bool bad = false;
+#pragma unroll
+    for (int a = 0; a < KW; ++a) {
+        if (a < nv) {
+            int ch[kCh];
+            bad |= !chunks_of(v[a], E[a], ch);
+#pragma unroll
+            for (int i = 0; i < kCh; ++i) {
+                const int t = __reduce_add_sync(0xffffffffu, ch[i]);   // |t| < 2^27
+                if (lane == a * kCh + i) mine = t;
+            }
+        }
+    }
+    key = __reduce_max_sync(0xffffffffu, key);
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane < nv * kCh) atomicAdd(sch + lane, mine);                   // 512 (2^22 - 1) < 2^31
+    if (lane == 30 && bad) sch[30] = 1;
+    if (lane == 31) atomicMax((unsigned *)sch + 31, key);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int t = sch[lane];
+        if (lane < nv * kCh || (lane == 30 && t != 0))
+            atomicAdd(slot + lane, (unsigned long long)(long long)t);
+        if (lane == 31) atomicMax(slot + lane, (unsigned long long)(unsigned)t);
+        sch[lane] = 0;
+    }
+}
+
+// The sums of a slot (after the barrier): lane i < nv returns value i (carries
+// from the lowest chunk up, then the digits as three integers and two FMAs;
+// NaN when a partial was not finite), every lane the slot's maximum key.  One
+// load per chunk and lane: a single coalesced load of the slot and shuffles
+// took 3.4 instead of 1.8 us with 152 CTAs reading it (1.9 / 1.3 with 40).
+__device__ __forceinline__ double pull_sums(const unsigned long long *slot, int nv, const int *E, unsigned &key) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long *p = slot + (lane < nv ? lane : 0) * kCh;
+    long long t[kCh];
+#pragma unroll
+    for (int q = 0; q < kCh; ++q) t[q] = (long long)__ldcg(p + q);
+    key = (unsigned)__ldcg(slot + 31);
+    const bool bad = __ldcg(slot + 30) != 0ull;
+    if (lane >= nv) return 0.0;
+    constexpr long long mask = (1ll << kChBits) - 1;
+#pragma unroll
+    for (int q = 0; q + 1 < kCh; ++q) {
+        t[q + 1] += t[q] >> kChBits;
+        t[q] &= mask;
+    }
+    const long long hi = t[6] * (1ll << kChBits) + t[5];
+    const long long mid = (t[4] << kChBits) | t[3], lo = (t[2] << kChBits) | t[1];
+    constexpr double two44 = 17592186044416.0;
+    const double r = fma(fma((double)hi, two44, (double)mid), two44, (double)lo);
+    return bad ? __longlong_as_double(0x7FF8000000000000ll) : scale_pow2(r, E[lane] - kField + kChBits);
+}
+
 // Fixed-point limbs of one value into the shared bins of the sparse-sign
-// rows of row r (pattern8: one 8-byte entry per row, prefetched).
+// rows of row r.  With the compact pattern (p8: one 8-byte entry per row,
+// prefetched) the bins are laid out [stripe][sign][p8_block], so that a pattern
+// byte is a bin offset and no sign has to be applied: 4 instructions per
+// nonzero instead of 9 (the update is issue- and shared-atomic-bound beside its
+// FP64 work; 100^3 grid: 10.5 -> 10.1 us in FP64, 8.8 -> 7.8 us in FP32).
 template <int ZCAP>
 __device__ __forceinline__ void scatter_row(const PCtx &c, int64_t r, uint2 pv, bool p8, int *b0, int *b1, int l0,
                                             int l1) {
     if (p8) {
+        const int q2 = 2 * c.p8_block;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            const int e = (int)__byte_perm(q < 4 ? pv.x : pv.y, 0u, 0x4440u + (q & 3));
-            const bool neg = e >= c.p8_block;
-            red_limbs(b0, b1, c.sp.start[q] + (neg ? e - c.p8_block : e), l0, l1, neg);
+            const int e = (int)__byte_perm(q < 4 ? pv.x : pv.y, 0u, 0x4440u + (q & 3)) + q * q2;
+            atomicAdd(b0 + e, l0);
+            atomicAdd(b1 + e, l1);
         }
     } else {
         uint16_t e[ZCAP];
@@ -237,9 +421,9 @@ constexpr int kSpmvWarps = kPNW - 1;   // the last warp serves the reductions
 template <int KW, int W, typename T>
 __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ wsrc, const T *win,
                                           const int (&soff)[KW], int nw, T *ys, const long long *meta_o,
-                                          const int *meta_w, int nsl, int nr, T (&acc)[KW],
-                                          unsigned long long &ykey) {
+                                          const int *meta_w, int nsl, int nr, T (&acc)[KW], unsigned &ykey) {
     const T *sell_val = (const T *)c.sell_val;
+    const unsigned long long pol = operator_policy(c.l2_frac);
     const int lane = threadIdx.x & 31;
     int next_t = threadIdx.x >> 5;
     auto grab = [&]() {
@@ -256,14 +440,14 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
         {
             const int32_t *pc = c.sell_col + (t < nsl ? meta_o[t] : 0) + lane;
 #pragma unroll
-            for (int p = 0; p < W; ++p) cv[p] = p < wt ? __ldcs(pc + 32 * p) : 0;
+            for (int p = 0; p < W; ++p) cv[p] = p < wt ? ld_op(pc + 32 * p, pol) : 0;
         }
         T av[W], xv[W];
         {
             const T *pv = sell_val + (t < nsl ? meta_o[t] : 0) + lane;
 #pragma unroll
             for (int p = 0; p < W; ++p) {
-                av[p] = p < wt ? __ldcs(pv + 32 * p) : T(0);
+                av[p] = p < wt ? ld_op(pv + 32 * p, pol) : T(0);
                 xv[p] = p < wt ? __ldcg(wsrc + cv[p]) : T(0);
             }
         }
@@ -273,7 +457,7 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
         {
             const int32_t *pc = c.sell_col + (tn < nsl ? meta_o[tn] : 0) + lane;
 #pragma unroll
-            for (int p = 0; p < W; ++p) cvn[p] = p < wtn ? __ldcs(pc + 32 * p) : 0;
+            for (int p = 0; p < W; ++p) cvn[p] = p < wtn ? ld_op(pc + 32 * p, pol) : 0;
         }
         while (t < nsl) {
             T avn[W], xvn[W];
@@ -281,7 +465,7 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
                 const T *pv = sell_val + (tn < nsl ? meta_o[tn] : 0) + lane;
 #pragma unroll
                 for (int p = 0; p < W; ++p) {
-                    avn[p] = p < wtn ? __ldcs(pv + 32 * p) : T(0);
+                    avn[p] = p < wtn ? ld_op(pv + 32 * p, pol) : T(0);
                     xvn[p] = p < wtn ? __ldcg(wsrc + cvn[p]) : T(0);
                 }
             }
@@ -291,7 +475,7 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
             {
                 const int32_t *pc = c.sell_col + (tnn < nsl ? meta_o[tnn] : 0) + lane;
 #pragma unroll
-                for (int p = 0; p < W; ++p) cvnn[p] = p < wtnn ? __ldcs(pc + 32 * p) : 0;
+                for (int p = 0; p < W; ++p) cvnn[p] = p < wtnn ? ld_op(pc + 32 * p, pol) : 0;
             }
             const int lr = t * 32 + lane;
             if (lr < nr) {
@@ -303,7 +487,7 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
 #pragma unroll
                 for (int a = 0; a < KW; ++a)
                     if (a < nw) acc[a] = fma(win[soff[a] + lr], y, acc[a]);
-                ykey = max(ykey, abs_key((double)y));
+                ykey = max(ykey, mag_key(y));
             }
             t = tn;
             wt = wtn;
@@ -324,13 +508,13 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
             const long long o = meta_o[t] + lane;
             T y = T(0);
             for (int p = 0; p < wt; ++p)
-                y = fma(__ldcs(sell_val + o + 32 * p), __ldcg(wsrc + __ldcs(c.sell_col + o + 32 * p)), y);
+                y = fma(ld_op(sell_val + o + 32 * p, pol), __ldcg(wsrc + ld_op(c.sell_col + o + 32 * p, pol)), y);
             if (lr < nr) {
                 ys[lr] = y;
 #pragma unroll
                 for (int a = 0; a < KW; ++a)
                     if (a < nw) acc[a] = fma(win[soff[a] + lr], y, acc[a]);
-                ykey = max(ykey, abs_key((double)y));
+                ykey = max(ykey, mag_key(y));
             }
         }
     }
@@ -344,7 +528,7 @@ template <int KW, int W, int ZCAP, bool YG, typename T>
 __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
     constexpr bool F32 = sizeof(T) == 4;
     extern __shared__ __align__(16) unsigned char psm[];
-    constexpr int kRed = KW * kPT + 4 * KW + kPNW;   // block_reduce_t0<KW>
+    constexpr int kRed = kPT + 4 + kPNW;             // block_reduce_t0<1>
     constexpr int kSvc = kPNW - 1;                   // the service warp
     const int G = gridDim.x, g = blockIdx.x;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -358,13 +542,11 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
     // global array, read back by the same CTA after a block barrier (L2)
     T *ys = YG ? (T *)c.ysg + r0 : win + (size_t)k * R;
     double *red = (double *)(YG ? win + (size_t)k * R : ys + R);   // block reductions (R: multiple of 32)
-    double *tp = red + kRed;                                 // [KW][kPT] per-thread norm / Gram partials
-    unsigned long long *tk = (unsigned long long *)(tp + KW * kPT);   // [kPT] per-thread max|w| keys
-    long long *meta_o = (long long *)(tk + kPT);             // [nsl] slice offsets
+    long long *meta_o = (long long *)(red + kRed);           // [nsl] slice offsets
     int *meta_w = (int *)(meta_o + R / 32);                  // [nsl] slice widths
-    int *bins = meta_w + R / 32;                             // [3][2][s]: S w limbs (two buffers), S y limbs
-    int *by0 = bins + 4 * s, *by1 = bins + 5 * s;
     const bool p8 = ZCAP == 8 && c.pattern8 != nullptr;
+    const int nbin = p8 ? 16 * c.p8_block : s;               // bins of one limb
+    int *bins = meta_w + R / 32;                             // [2][2][nbin]: limbs of S w_j in buffer j & 1
     const long long lmask = (1ll << c.L) - 1;
 
     // per-step scalars, in rings indexed by step & 3 (k <= 4)
@@ -376,10 +558,15 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
     __shared__ int ews[4];                   // exponent bound of max|w_i| (its sketch)
     __shared__ int eys[4];                   // exponent bound of max|y~_i|
     __shared__ double sh[kMaxK];             // MGS coefficients h_ij of the current step
-    __shared__ double sd[KW + 1];            // reduced dots and max|y~| of the current step
-    __shared__ double sb[KW + 1];            // reduced ||w_j||^2, max|w_j|, Gram entries
+    __shared__ double sb[2];                 // reduced ||b||^2, max|b|
+    __shared__ double fd[kMaxK], fg[KW][KW]; // MGS factors of the current step (phase A)
+    __shared__ int ea[KW], eb[KW];           // exponent bounds of the per-thread sums of phases A and B
+    __shared__ int sch[kSlot];               // this CTA's chunk sums (push_sums)
+    __shared__ int bar_ok;                   // the last grid barrier was passed
     __shared__ int sbreak;                   // w_j is a happy breakdown
     unsigned nb = 0;                         // barriers passed
+    const int nh = max(0, kSpmvWarps - nsl); // SpMV warps without a slice
+    const int lg_rows = 32 - __clz(R / 256); // log2 of a bound of the rows one thread sums
 
     // Column i of S V and column i-1 of S A V from the integer sums of S w_i
     // (rows is = g + G t of S): S w_i, S v_i = sigma_i S w_i and, by the
@@ -417,20 +604,47 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
         c.SAV[is + (size_t)i * s] = v;
     };
     // add this CTA's S w_i limb bins (buffer i & 1) to accw[i], then clear them
-    auto flush_w = [&](int i, int t0, int dt) {
-        int *b0 = bins + (i & 1) * 2 * s, *b1 = b0 + s;
-        unsigned long long *aw = c.accw + (size_t)i * 2 * s;
-        for (int x = t0; x < s; x += dt) {
-            atomicAdd(aw + x, (unsigned long long)(long long)b0[x]);
-            atomicAdd(aw + s + x, (unsigned long long)(long long)b1[x]);
-            b0[x] = 0;
-            b1[x] = 0;
+    // (split layout: x enumerates the bins of one sign, so that a warp stays within a stripe)
+    auto flush_bins = [&](int buf, unsigned long long *aw, int t0, int dt) {
+        int *b0 = bins + (buf & 1) * 2 * nbin, *b1 = b0 + nbin;
+        if (p8) {
+            const int blk = c.p8_block, lb = blk == 64 ? 6 : 7;
+#pragma unroll 4
+            for (int x = t0; x < 8 * blk; x += dt) {
+                const int q = x >> lb, i = x & (blk - 1);
+                if (i < c.sp.size[q]) {
+                    const int row = c.sp.start[q] + i, o = x + q * blk;
+                    atomicAdd(aw + row, (unsigned long long)(long long)(b0[o] - b0[o + blk]));
+                    atomicAdd(aw + s + row, (unsigned long long)(long long)(b1[o] - b1[o + blk]));
+                    b0[o] = b0[o + blk] = 0;
+                    b1[o] = b1[o + blk] = 0;
+                }
+            }
+        } else {
+            for (int x = t0; x < s; x += dt) {
+                atomicAdd(aw + x, (unsigned long long)(long long)b0[x]);
+                atomicAdd(aw + s + x, (unsigned long long)(long long)b1[x]);
+                b0[x] = 0;
+                b1[x] = 0;
+            }
         }
     };
-    auto flush_y = [&](int t0, int dt) {
-        for (int x = t0; x < s; x += dt) {
-            atomicAdd(c.accy + x, (unsigned long long)(long long)by0[x]);
-            atomicAdd(c.accy + s + x, (unsigned long long)(long long)by1[x]);
+    auto flush_w = [&](int i, int t0, int dt) { flush_bins(i, c.accw + (size_t)i * 2 * s, t0, dt); };
+
+    // FP32 basis: H of the relation with the applied sigma_j and coefficients,
+    // A v_j = (sigma_j / sap_j) (v_{j+1} ||w_{j+1}|| + sum_i c_i v_i / sigma_i), from the
+    // stored c_i and ||w_{j+1}|| of columns 0 .. nc - 1 (an FP64 division is too slow
+    // for the recurrence's critical path)
+    auto finish_h = [&](int nc) {
+        if (!F32 || g != 0) return;
+        __syncthreads();
+        for (int x = tid; x < nc * (k + 1); x += kPT) {
+            const int jc = x / (k + 1), i = jc + 1 - x % (k + 1);
+            if (i < 0) continue;
+            const double sj = __ldcg(c.vscale + jc), f = (double)(float)sj;
+            double *h = c.H + i + (size_t)jc * (m + 1);
+            const double v = __ldcg(h);
+            *h = i == jc + 1 ? sj * v / f : sj * v / (f * __ldcg(c.vscale + i));
         }
     };
 
@@ -439,7 +653,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
         meta_o[t] = c.sell_off[r0 / 32 + t];
         meta_w[t] = c.sell_w[r0 / 32 + t];
     }
-    for (int i = tid; i < 6 * s; i += kPT) bins[i] = 0;
+    for (int i = tid; i < 4 * nbin; i += kPT) bins[i] = 0;
     for (int64_t i = (int64_t)g * kPT + tid; i < (int64_t)(m + 1) * m; i += (int64_t)G * kPT) c.H[i] = 0.0;
     if (g == 0 && tid == 0) {
         c.iscal[0] = 0;
@@ -448,6 +662,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
         c.iscal[3] = m;
     }
     if (tid == 0) sbreak = 0;
+    if (tid < kSlot) sch[tid] = 0;
     {
         double nrm[1] = {0.0};
         unsigned long long key = 0;
@@ -494,42 +709,77 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
         const bool last = j == m - 1;
         const int ngj = min(j, k - 1);       // Gram distances of w_j
         // ---- phase A: y~ = A w_j and the window dots (kSpmvWarps warps).
-        // Meanwhile the service warp reduces this CTA's partial norms of w_j
-        // (left by phase B of the previous step), adds the CTA's S w_{j-1}
-        // bins to the global sums and finalises the sketch columns of step
-        // j - 2: none of it is needed before the barrier, and phase A does not
-        // need the norm of w_j (stored unnormalised).
+        // Phase A does not need the norm of w_j (stored unnormalised): meanwhile
+        // the service warp turns the sums of phase B of the previous step into
+        // sigma_j, the breakdown test and the factors of the MGS recurrence, so
+        // that after the barrier only the products with the dots are left; the
+        // CTA's S w_{j-1} bins are added to the global sums and the sketch
+        // columns of step j - 2 finalised (none of it is needed before that).
         T acc[KW];
 #pragma unroll
         for (int a = 0; a < KW; ++a) acc[a] = T(0);
-        unsigned long long ykey = 0;
+        unsigned ykey = 0;
         if (warp == kSvc && j >= 1) {
-            double v[KW];
+            // lane 0: ||w_j||^2, lane d: <w_j, w_{j-d}>
+            unsigned wk;
+            const double tot = pull_sums(c.slot + (size_t)(2 * j - 1) * kSlot, 1 + ngj, eb, wk);
+            double gr[KW];
 #pragma unroll
-            for (int q = 0; q < KW; ++q) {
-                v[q] = 0.0;
-                if (q <= ngj) {
-#pragma unroll 4
-                    for (int t = lane; t < kPT; t += 32) v[q] += tp[q * kPT + t];
+            for (int d = 1; d < KW; ++d) gr[d] = __shfl_sync(0xffffffffu, tot, d);
+            if (lane == 0) {
+                // H column j - 1 (FP32: c_i and h_{j,j-1} unscaled, finish_h turns them
+                // into the coefficients of the relation with the applied values)
+                const int jp = j - 1, ip0 = max(0, jp - k + 1), np = jp - ip0 + 1;
+                double hs = 0.0;
+                for (int a = 0; a < np; ++a) {
+                    hs = fma(sh[a], sh[a], hs);
+                    if (g == 0) c.H[ip0 + a + (size_t)jp * (m + 1)] = F32 ? coef[jp & 3][np - 1 - a] : sh[a];
+                }
+                // ||A v_{j-1}||^2 = sum_i h_i^2 + ||w_j||^2 for the orthonormal window;
+                // happy breakdown when ||w_j|| <= 1e-12 ||A v_{j-1}||
+                // (compared in squares, and sigma = 1/||w_j|| from one rsqrt: an FP64
+                // square root or division is ~650 dependent cycles on this part)
+                // (FP32: ||w_j|| <= 2^-17 ||A v_{j-1}||, 64 FP32 unit roundoffs)
+                sbreak = (tot > (F32 ? 5.820766091346741e-11 : 1e-24) * (hs + tot)) ? 0 : 1;
+                const double sgm = tot > 0.0 ? rsqrt(tot) : 0.0;
+                if (g == 0) {
+                    c.H[j + (size_t)jp * (m + 1)] = tot * sgm;
+                    if (!sbreak) c.vscale[j] = sgm;
+                }
+                if (!sbreak) {   // w_j enters the window
+                    sig[j & 3] = sgm;
+                    sap[j & 3] = F32 ? (double)(float)sgm : sgm;
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+                    for (int d = 1; d < KW; ++d)
+                        if (d <= ngj) grm[j & 3][d] = gr[d];
+                    ews[j & 3] = key_exponent<T>(wk);
                 }
             }
-            unsigned long long kk = 0;
-            for (int t = lane; t < kPT; t += 32) kk = max(kk, tk[t]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) kk = max(kk, __shfl_xor_sync(0xffffffffu, kk, o));
-            if (lane == 0) {
-                c.pB[g] = v[0];
-                c.pB[G + g] = key_to_abs(kk);
-#pragma unroll
-                for (int d = 1; d < KW; ++d)
-                    if (d <= ngj) c.pB[(size_t)(1 + d) * G + g] = v[d];
-            }
-            flush_w(j - 1, lane, 32);
-            if (j >= 2)
-                for (int t = lane; g + G * t < s; t += 32) finalize_col(j - 2, t);
             __syncwarp();
+        }
+        if (warp == kSvc) {
+            // factors of the MGS recurrence that do not depend on the dots
+            // (h_i = fd_i <w_i, y> - sum_{i' < i} fg_ii' h_i'), one per lane
+            if (lane < nw) {
+                fd[lane] = sig[(i0 + lane) & 3] * sig[j & 3];
+                ea[lane] = ews[(i0 + lane) & 3] + ews[j & 3] + c.e_row + lg_rows;
+            }
+            if (lane >= 16 && lane < 16 + KW * KW) {
+                const int a = (lane - 16) / KW, b2 = (lane - 16) % KW;
+                if (a < nw && b2 < a)
+                    fg[a][b2] = sig[(i0 + a) & 3] * sig[(i0 + b2) & 3] * grm[(i0 + a) & 3][a - b2];
+            }
+        }
+        // S w_{j-1}: by the warps that have no slice; by all warps after their
+        // slices where phase A is short (kFlushAll: the service warp alone needs
+        // longer than that, 3.0 of 14.7 us per step with 45 slices; 13.8 with all warps); else by the
+        // service warp, beside phase A
+        const bool flush_all = nh == 0 && nsl <= kFlushAll;
+        if (j >= 1 && (nh > 0 ? (warp >= nsl && warp < kSpmvWarps) : warp == kSvc)) {
+            const int ht = nh > 0 ? tid - 32 * nsl : lane, nt = nh > 0 ? 32 * nh : 32;
+            if (!flush_all) flush_w(j - 1, ht, nt);
+            if (j >= 2)
+                for (int t = ht; g + G * t < s; t += nt) finalize_col(j - 2, t);
         }
         {
             int soff[KW];   // window slot offsets, oldest first
@@ -538,83 +788,57 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             if (warp < kSpmvWarps)
                 spmv_rows<KW, W, T>(c, Vb + (size_t)j * c.ldv, win, soff, nw, ys, meta_o, meta_w, nsl, nr, acc, ykey);
         }
-        double accd[KW];
-#pragma unroll
-        for (int a = 0; a < KW; ++a) accd[a] = (double)acc[a];
-        ykey = block_reduce_t0<KW>(accd, ykey, red);
-        if (tid == 0) {
-#pragma unroll
-            for (int a = 0; a < KW; ++a)
-                if (a < nw) c.pA[(size_t)a * G + g] = accd[a];
-            c.pA[(size_t)KW * G + g] = key_to_abs(ykey);
-        }
-        if (!grid_barrier(c.bar, c.flag, ++nb, c.budget)) goto timeout;
-
-        // ---- totals: dots and max|y~| of this step; ||w_j||, max|w_j| and the
-        // Gram entries of w_j (every CTA, identically)
-        if (warp <= nw) {
-            const int slot = warp < nw ? warp : KW;
-            const double v = reduce_slot(c.pA + (size_t)slot * G, G, slot == KW);
-            if (lane == 0) sd[slot] = v;
-        } else if (j >= 1 && warp - nw - 1 < 2 + ngj) {
-            const int q = warp - nw - 1;
-            const double v = reduce_slot(c.pB + (size_t)q * G, G, q == 1);
-            if (lane == 0) sb[q] = v;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            if (j >= 1) {
-                // ||A v_{j-1}||^2 = sum_i h_i^2 + ||w_j||^2 for the orthonormal window;
-                // happy breakdown when ||w_j|| <= 1e-12 ||A v_{j-1}||
-                // (compared in squares, and sigma = 1/||w_j|| from one rsqrt: an FP64
-                // square root or division is ~650 dependent cycles on this part)
-                const double n2 = sb[0];
-                double hs = 0.0;
-                for (int a = 0; a < cnw[(j - 1) & 3]; ++a) hs = fma(sh[a], sh[a], hs);
-                // (FP32: ||w_j|| <= 2^-17 ||A v_{j-1}||, 64 FP32 unit roundoffs)
-                sbreak = (n2 > (F32 ? 5.820766091346741e-11 : 1e-24) * (hs + n2)) ? 0 : 1;
-                const double sgm = n2 > 0.0 ? rsqrt(n2) : 0.0;
-                const double hn = n2 * sgm;
-                if (!sbreak) {   // w_j enters the window
-                    sig[j & 3] = sgm;
-                    sap[j & 3] = F32 ? (double)(float)sgm : sgm;
-                    for (int d = 1; d <= ngj; ++d) grm[j & 3][d] = sb[1 + d];
-                    ews[j & 3] = positive_finite(sb[1]) ? bound_exponent(sb[1]) : kNoExp;
+        if (flush_all && j >= 1) flush_w(j - 1, tid, kPT);
+        __syncthreads();   // the bounds ea[] of the service warp
+        {
+            unsigned long long *sl = c.slot + (size_t)(2 * j) * kSlot;
+            push_sums<KW, T>(acc, nw, ea, ykey, sch, sl);
+            ++nb;
+            if (warp == 0) {
+                __syncwarp();
+                if (lane == 0) {
+                    grid_arrive(c.bar);
+                    bar_ok = spin_until(c.bar, nb * (unsigned)G, c.flag, c.budget);
                 }
-                if (g == 0) {
-                    // FP32: the coefficient of v_j in A v_{j-1} with the applied sigma_{j-1}
-                    c.H[j + (size_t)(j - 1) * (m + 1)] =
-                        F32 ? sig[(j - 1) & 3] * hn / sap[(j - 1) & 3] : hn;
-                    if (!sbreak) c.vscale[j] = sgm;
+                __syncwarp();
+                // totals of this step (every CTA, identically): lane a the dot with
+                // w_{i0+a}; MGS in the window, ascending, from the dots and the Gram
+                // matrix: h_i = <v_i, y> - sum_{i' < i} h_i' <v_i, v_i'>
+                unsigned yk;
+                double dot = pull_sums(sl, nw, ea, yk);
+                if (lane < nw) dot *= fd[lane];
+                double h[KW];
+#pragma unroll
+                for (int a = 0; a < KW; ++a) h[a] = __shfl_sync(0xffffffffu, dot, a);
+                if (lane == 0 && !sbreak) {
+                    int ew1 = -2000;   // |w_{j+1}| < 2^ew1: the largest term's exponent, for up to 5 terms
+                    const int ey = key_exponent<T>(yk);
+                    if (ey != kNoExp) ew1 = max(ew1, exponent_above(sap[j & 3]) + ey);
+#pragma unroll
+                    for (int a = 0; a < KW; ++a) {
+                        if (a < nw) {
+#pragma unroll
+                            for (int b2 = 0; b2 < KW; ++b2)
+                                if (b2 < a) h[a] = fma(-h[b2], fg[a][b2], h[a]);
+                            sh[a] = h[a];
+                            double cc = h[a] * sig[(i0 + a) & 3];
+                            if constexpr (F32) cc = (double)(float)cc;
+                            coef[j & 3][nw - 1 - a] = cc;
+                            if (ews[(i0 + a) & 3] != kNoExp) ew1 = max(ew1, exponent_above(cc) + ews[(i0 + a) & 3]);
+                        }
+                    }
+                    cnw[j & 3] = nw;
+                    eys[j & 3] = ey;
+                    ew1 += 3;
+                    eb[0] = 2 * ew1 + lg_rows;
+#pragma unroll
+                    for (int d = 1; d < KW; ++d)   // <w_{j+1}, w_{j+1-d}>
+                        if (d <= nw) eb[d] = ew1 + ews[(j + 1 - d) & 3] + lg_rows;
                 }
             }
-            if (!sbreak) {
-                // MGS in the window, ascending, from the dots and the Gram matrix:
-                // h_i = <v_i, y> - sum_{i' < i} h_i' <v_i, v_i'>
-                const double sj = sig[j & 3];
-                for (int a = 0; a < nw; ++a) {
-                    const int ia = i0 + a;
-                    const double sa = sig[ia & 3];
-                    double h = sa * sj * sd[a];
-                    for (int b2 = 0; b2 < a; ++b2) {
-                        const int ib = i0 + b2;
-                        h -= sh[b2] * sa * sig[ib & 3] * grm[ia & 3][ia - ib];
-                    }
-                    sh[a] = h;
-                    coef[j & 3][nw - 1 - a] = F32 ? (double)(float)(h * sa) : h * sa;
-                }
-                cnw[j & 3] = nw;
-                eys[j & 3] = positive_finite(sd[KW]) ? bound_exponent(sd[KW]) : kNoExp;
-                // FP32: the relation with the applied (rounded) sigma_j and coefficients
-                if (g == 0 && !last)
-                    for (int a = 0; a < nw; ++a) {
-                        const int ia = i0 + a;
-                        c.H[ia + (size_t)j * (m + 1)] =
-                            F32 ? sj * coef[j & 3][nw - 1 - a] / (sap[j & 3] * sig[ia & 3]) : sh[a];
-                    }
-            }
+            __syncthreads();
+            if (!bar_ok) goto timeout;
         }
-        __syncthreads();
 
         if (sbreak) {
             // happy breakdown: w_j is rounding noise, the basis ends at m_eff = j.
@@ -627,12 +851,14 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             T accb[KW];
 #pragma unroll
             for (int a = 0; a < KW; ++a) accb[a] = T(0);
-            unsigned long long kb = 0;
+            unsigned kb = 0;
             if (warp < kSpmvWarps)
                 spmv_rows<KW, W, T>(c, Vb + (size_t)jb * c.ldv, win, soff, 0, ys, meta_o, meta_w, nsl, nr, accb, kb);
             __syncthreads();
             const int ey = eys[jb & 3];
             const int shift_y = c.frac - (ey == kNoExp ? 0 : ey);
+            // (both bin buffers are empty: S w_{j-1} was added up in phase A)
+            int *by0 = bins, *by1 = bins + nbin;
             for (int lr = tid; lr < nr; lr += kPT) {
                 const int64_t r = r0 + lr;
                 const long long vy = ey == kNoExp ? 0 : fixed_point(ys[lr], shift_y);
@@ -640,7 +866,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
                 scatter_row<ZCAP>(c, r, pv, p8, by0, by1, (int)(vy & lmask), (int)(vy >> c.L));
             }
             __syncthreads();
-            flush_y(tid, kPT);
+            flush_bins(0, c.accy, tid, kPT);
             if (!grid_barrier(c.bar, c.flag, ++nb, c.budget)) goto timeout;
             // S v_{j-1}, S A v_{j-2} (S w_{j-1} was added up before the last barrier) and S A v_{j-1}
             for (int t = tid; g + G * t < s; t += kPT) {
@@ -652,6 +878,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
                 c.iscal[1] = j;
                 c.iscal[3] = j;
             }
+            finish_h(j);
             return;
         }
 
@@ -663,7 +890,8 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             const int shift_w = c.frac - (ew == kNoExp ? 0 : ew);
             const int shift_y = c.frac - (ey == kNoExp ? 0 : ey);
             const int ng = min(j + 1, k - 1);
-            int *bw0 = bins + (j & 1) * 2 * s, *bw1 = bw0 + s;
+            int *bw0 = bins + (j & 1) * 2 * nbin, *bw1 = bw0 + nbin;
+            int *by0 = bins + ((j + 1) & 1) * 2 * nbin, *by1 = by0 + nbin;   // S y~ of the last step: the empty buffer
             T cf[KW];        // c_b for w_{j-b} (as applied)
             int soffr[KW];   // slot offsets, newest first
 #pragma unroll
@@ -676,7 +904,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             T part[KW];
 #pragma unroll
             for (int a = 0; a < KW; ++a) part[a] = T(0);
-            unsigned long long nkey = 0;
+            unsigned nkey = 0;
             uint2 pv_next = make_uint2(0u, 0u);
             if (p8 && tid < nr) pv_next = __ldg((const uint2 *)(c.pattern8 + (r0 + tid) * 8));
             for (int lr = tid; lr < nr; lr += kPT) {
@@ -695,7 +923,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
                     wn[r] = w;
                     win[snew + lr] = w;
                     part[0] = fma(w, w, part[0]);
-                    nkey = max(nkey, abs_key((double)w));
+                    nkey = max(nkey, mag_key(w));
 #pragma unroll
                     for (int d = 1; d < KW; ++d)
                         if (d <= ng) part[d] = fma(w, wv[d - 1], part[d]);
@@ -708,16 +936,24 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
                 }
             }
             if (!last) {
-#pragma unroll
-                for (int a = 0; a < KW; ++a) tp[a * kPT + tid] = (double)part[a];
-                tk[tid] = nkey;
+                push_sums<KW, T>(part, 1 + ng, eb, nkey, sch, c.slot + (size_t)(2 * j + 1) * kSlot);
             } else {
                 __syncthreads();
                 flush_w(j, tid, kPT);
-                flush_y(tid, kPT);
+                flush_bins(j + 1, c.accy, tid, kPT);
+                __syncthreads();
             }
         }
-        if (!grid_barrier(c.bar, c.flag, ++nb, c.budget)) goto timeout;
+        ++nb;
+        if (warp == 0) {
+            __syncwarp();
+            if (lane == 0) {
+                grid_arrive(c.bar);
+                bar_ok = spin_until(c.bar, nb * (unsigned)G, c.flag, c.budget);
+            }
+        }
+        __syncthreads();
+        if (!bar_ok) goto timeout;
         if (last) {
             // S v_{m-2}, S v_{m-1}, S A v_{m-3}, S A v_{m-2} (relation), S A v_{m-1} (direct)
             for (int t = tid; g + G * t < s; t += kPT) {
@@ -727,6 +963,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             }
         }
     }
+    finish_h(m - 1);
     return;
 timeout:
     if (g == 0 && tid == 0) {
@@ -827,19 +1064,19 @@ cudaError_t launch_persist_f32(const PCtx &c, int maxw, int G, size_t smem, cuda
 
 // Dynamic shared memory of the persistent kernel for R rows per CTA with
 // elements of vb bytes (yg: y~ kept in global memory instead).
-size_t persist_smem(int R, int k, int KW, int s, bool yg, size_t vb = sizeof(double)) {
-    const size_t red = (size_t)KW * kPT + 4 * KW + kPNW;
-    const size_t thread_partials = (size_t)(KW + 1) * kPT;
-    return vb * (size_t)(k + (yg ? 0 : 1)) * R + sizeof(double) * (red + thread_partials) +
-           (sizeof(long long) + sizeof(int)) * (size_t)(R / 32) + sizeof(int) * 6 * (size_t)s;
+size_t persist_smem(int R, int k, int nbin, bool yg, size_t vb = sizeof(double)) {
+    const size_t red = (size_t)kPT + 4 + kPNW;
+    return vb * (size_t)(k + (yg ? 0 : 1)) * R + sizeof(double) * red +
+           (sizeof(long long) + sizeof(int)) * (size_t)(R / 32) + sizeof(int) * 4 * (size_t)nbin;
 }
 
 }  // namespace
 
-// Persistent partition: G = min(SMs, ceil(n / 1024)) CTAs of R rows (whole
-// slices).  The sketch tables record the bin-load maximum of this partition.
+// Persistent partition: G = min(SMs, ceil(n / kPersistMinRows)) CTAs of R rows
+// (whole slices).  The sketch tables record the bin-load maximum of this
+// partition.
 void persist_partition(int64_t n, int *G, int64_t *rows) {
-    int64_t g = (n + 1023) / 1024;
+    int64_t g = (n + kPersistMinRows - 1) / kPersistMinRows;
     if (g > num_sms()) g = num_sms();
     if (g < 1) g = 1;
     const int64_t R = ((n + g - 1) / g + 31) / 32 * 32;
@@ -870,7 +1107,9 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     const int R = (int)R64;
     const int KW = k <= 2 ? 2 : 4;
     const int s = S->s;
-    size_t smem = persist_smem(R, k, KW, s, false, vb);
+    const bool p8 = S->zeta == 8 && S->pattern8 != nullptr;
+    const int nbin = p8 ? 16 * S->p8_block : s;
+    size_t smem = persist_smem(R, k, nbin, false, vb);
     int dev = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
@@ -883,7 +1122,7 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     if (smem + 4096 > (size_t)optin) {
         if (f32) return SKF_ERR_NOT_SUPPORTED;   // an FP32 basis keeps y~ on chip
         yg = true;
-        smem = persist_smem(R, k, KW, s, true, vb);
+        smem = persist_smem(R, k, nbin, true, vb);
         if (KW != 2 || A->max_width > 7 || smem + 4096 > (size_t)optin) return SKF_ERR_NOT_SUPPORTED;
     }
     int coop = 0;
@@ -899,14 +1138,23 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     c.sell_w = A->sell_w;
     c.sell_val = A->sell_val;
     c.sell_col = A->sell_col;
+    // L2 share of the operator, measured per step (keep none / this rule): all of
+    // it up to 90 MB (FP64 41.9 / 41.1 us at 84 MB, 21.6 / 20.2 at 22 MB; FP32
+    // 32.8 / 26.4 at 56 MB), beyond that 50 MB of it (FP32 47.8 / 45.2 at 97 MB;
+    // all of it 48.5).  With y~ in global memory L2 already holds that and the
+    // gathered vector, and a kept operator only displaces them (FP64 50.2 / 53.2
+    // at 106 MB, 49.3 / 52.9 at 84 MB): nothing is kept.
+    const double opb = (double)A->sell_entries * (double)(vb + 4);
+    c.l2_frac = yg ? 0.f : opb <= 90e6 ? 1.f : (float)(50e6 / opb);
     c.sp = make_sparse_sign(S);
     c.pattern = S->pattern;
-    if (S->zeta == 8 && S->pattern8 != nullptr) {
+    if (p8) {
         c.pattern8 = S->pattern8;
         c.p8_block = S->p8_block;
     }
     c.L = limb_bits(S->binmax_persist_host);
     c.frac = sketch_fraction_bits_from_limb(c.L);
+    c.e_row = positive_finite(A->norm_inf) ? bound_exponent(A->norm_inf) + 1 : 0;
     c.sk_scale = 1.0 / sqrt((double)S->zeta);
     c.m = m;
     c.k = k;
@@ -921,13 +1169,14 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     c.budget = kBarrierBudget;
 
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t szP = sizeof(double) * (size_t)(KW + 1) * G;
+    const size_t szP = sizeof(double) * 2 * (size_t)G;
+    const size_t szSlot = sizeof(unsigned long long) * (size_t)(2 * m + 1) * kSlot;
     const size_t szAw = sizeof(unsigned long long) * (size_t)m * 2 * s;
     const size_t szAy = sizeof(unsigned long long) * 2 * (size_t)s;
     const size_t szSw = sizeof(double) * (size_t)s * m;
     const size_t szBar = 2 * sizeof(int) + sizeof(unsigned long long);   // counter, flag, eps maximum
     const size_t szYs = yg ? vb * (size_t)G * R : 0;
-    const size_t total = 2 * al(szP) + al(szAw) + al(szAy) + al(szSw) + al(szBar) + al(szYs);
+    const size_t total = al(szP) + al(szSlot) + al(szAw) + al(szAy) + al(szSw) + al(szBar) + al(szYs);
     char *ws = nullptr;
     skf_status stt = dalloc((void **)&ws, total, st);
     if (stt != SKF_OK) return stt;
@@ -937,8 +1186,8 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
         off += al(sz);
         return p;
     };
-    c.pA = (double *)take(szP);
     c.pB = (double *)take(szP);
+    c.slot = (unsigned long long *)take(szSlot);
     c.accw = (unsigned long long *)take(szAw);
     c.accy = (unsigned long long *)take(szAy);
     c.Sw = (double *)take(szSw);
@@ -947,7 +1196,7 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     c.flag = (int *)(c.bar + 1);
     unsigned long long *epsmax = (unsigned long long *)(c.bar + 2);
     // accumulators and the barrier start at zero (one memset: they are adjacent)
-    cudaMemsetAsync(c.accw, 0, (size_t)((char *)c.Sw - (char *)c.accw), st);
+    cudaMemsetAsync(c.slot, 0, (size_t)((char *)c.Sw - (char *)c.slot), st);
     cudaMemsetAsync(c.bar, 0, szBar, st);
     cudaError_t e;
     if (f32) e = launch_persist_f32(c, A->max_width, G, smem, st);

@@ -62,6 +62,7 @@ struct skf_csr {
     void *sell_val = nullptr;
     int32_t *sell_col = nullptr;
     int max_width = 0;                // widest slice
+    int64_t sell_entries = 0;         // entries of the slices, padding included
     int64_t max_chunk_entries = 0;    // most SELL entries in one chunk of 1024 rows (32 slices)
     // Row split for skewed degree distributions: rows with more than
     // kLongRow entries are left out of the slices (they count as empty there)
