@@ -69,6 +69,37 @@ __device__ __forceinline__ void load_pattern(const uint16_t *pattern, int zeta, 
     }
 }
 
+// Sketch of one value of a row with the compact pattern (zeta = 8): its limbs
+// into bins laid out [limb][stripe][sign][BLK] in 1 << LC copies (copy index in
+// the low bits, the caller's lane in `base`, a shared-memory address), so that a
+// pattern byte is a bin offset and everything else an immediate: four
+// instructions per nonzero.  The kernels that scatter are bound by instruction
+// issue or by these atomics, not by memory.
+template <int OFF>
+__device__ __forceinline__ void red_shared(unsigned addr, int v) {
+    asm volatile("red.shared.add.s32 [%0+%2], %1;" ::"r"(addr), "r"(v), "n"(OFF));
+}
+template <int BLK, int LC, int Q = 0>
+__device__ __forceinline__ void scatter8(uint2 pv, unsigned base, int l0, int l1) {
+    if constexpr (Q < 8) {
+        const unsigned e = __byte_perm(Q < 4 ? pv.x : pv.y, 0u, 0x4440u + (Q & 3));
+        const unsigned a = base + (e << (LC + 2));
+        red_shared<(Q * 2 * BLK) << (LC + 2)>(a, l0);
+        red_shared<((Q * 2 + 16) * BLK) << (LC + 2)>(a, l1);
+        scatter8<BLK, LC, Q + 1>(pv, base, l0, l1);
+    }
+}
+// one limb only
+template <int BLK, int LC, int Q = 0>
+__device__ __forceinline__ void scatter8_one(uint2 pv, unsigned base, int l0) {
+    if constexpr (Q < 8) {
+        const unsigned e = __byte_perm(Q < 4 ? pv.x : pv.y, 0u, 0x4440u + (Q & 3));
+        red_shared<(Q * 2 * BLK) << (LC + 2)>(base + (e << (LC + 2)), l0);
+        scatter8_one<BLK, LC, Q + 1>(pv, base, l0);
+    }
+}
+__device__ __forceinline__ unsigned shared_address(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
 // Arrival ticket: true in exactly one CTA, the last to finish its partials.
 __device__ __forceinline__ bool last_to_arrive(unsigned *cnt) {
     __shared__ bool last;
