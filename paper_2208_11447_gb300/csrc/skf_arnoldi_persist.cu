@@ -388,14 +388,10 @@ __device__ __forceinline__ double pull_sums(const unsigned long long *slot, int 
 template <int ZCAP>
 __device__ __forceinline__ void scatter_row(const PCtx &c, int64_t r, uint2 pv, bool p8, int *b0, int *b1, int l0,
                                             int l1) {
-    if (p8) {
-        const int q2 = 2 * c.p8_block;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int e = (int)__byte_perm(q < 4 ? pv.x : pv.y, 0u, 0x4440u + (q & 3)) + q * q2;
-            atomicAdd(b0 + e, l0);
-            atomicAdd(b1 + e, l1);
-        }
+    if (p8) {   // (b1 follows b0 by 16 p8_block bins)
+        const unsigned base = shared_address(b0);
+        if (c.p8_block == 64) scatter8<64, 0>(pv, base, l0, l1);
+        else scatter8<128, 0>(pv, base, l0, l1);
     } else {
         uint16_t e[ZCAP];
         load_pattern<ZCAP>(c.pattern, c.sp.zeta, r, e);
