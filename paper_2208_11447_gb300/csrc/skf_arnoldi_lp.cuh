@@ -99,18 +99,19 @@ __device__ __forceinline__ unsigned abs_key_f32(float x) { return __float_as_uin
 // l0 = rint((t - l1) 2^L) (the fractional part of a non-negative float is
 // exact); both limbs carry the sign of x.  0 <= |l0| <= 2^L, which keeps the
 // bin sums within the limb-width rule.  Requires |x| 2^shift < 2^(2L).  The
-// scales come from LimbScale, set once per kernel.
+// scales come from LimbScale, set once per kernel (the exponent in two halves,
+// so that no branch on its range is left in the row loop).
 struct LimbScale {
-    float hi, lo;   // 2^(shift - L) (0 if outside the float range), 2^L
-    int k;          // shift - L
+    float a, b, lo;   // a b = 2^(shift - L) (each a normal power of two), 2^L
     __device__ __forceinline__ LimbScale(int shift, int L) {
-        k = shift - L;
-        hi = (k >= -126 && k <= 127) ? __int_as_float((127 + k) << 23) : 0.f;
+        const int k = min(max(shift - L, -252), 254), h = k / 2;
+        a = __int_as_float((127 + h) << 23);
+        b = __int_as_float((127 + k - h) << 23);
         lo = __int_as_float((127 + L) << 23);
     }
 };
 __device__ __forceinline__ void limbs_f32(float x, const LimbScale &ls, int &l0, int &l1) {
-    const float t = ls.hi != 0.f ? fabsf(x) * ls.hi : ldexpf(fabsf(x), ls.k);
+    const float t = fabsf(x) * ls.a * ls.b;   // exact, or below one unit of limb 1 and of its fraction
     const float fl = floorf(t);
     const int h = __float2int_rz(fl);
     const int lo = __float2int_rn((t - fl) * ls.lo);
@@ -127,6 +128,7 @@ struct LpCtx {
     const int32_t *sell_w;
     const float *sell_val;
     const int32_t *sell_col;
+    int max_width;             // widest SELL slice
     double norm_inf;           // ||A||_inf
     SparseSign sp;
     const uint16_t *pattern;   // 16-bit sparse-sign pattern
@@ -506,13 +508,14 @@ __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv_lp(LpCtx c, in
     spmv_end<KW>(c, j, nw, last, L, bins, acc, ykey, red);
 }
 
-// Pipelined SpMV for operators whose SELL slices are at most 8 wide.  Chunk i
+// Pipelined SpMV for operators whose SELL slices are at most W <= 8 wide (W
+// product slots per row).  Chunk i
 // of the CTA is in three stages at once: its values and gathers are loaded
 // (the gathers use column indices loaded one iteration earlier), the column
 // indices of chunk i + 1 are loaded, and the slice width and offset of chunk
 // i + 2 are loaded.  One memory round trip per chunk instead of two (column,
 // then gather), with 8 extra registers per thread.
-template <int KW, int ZCAP, typename TB>
+template <int KW, int ZCAP, typename TB, int W>
 __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv_lp_pipe(LpCtx c, int j) {
     extern __shared__ int bins[];   // [2 s]: limbs of S w_j (stopping step) or of S y_{m-1} (last step)
     __shared__ double red[32 * KW];
@@ -541,71 +544,71 @@ __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv_lp_pipe(LpCtx 
 #pragma unroll
     for (int a = 0; a < KW; ++a) acc[a] = 0.f;
     unsigned ykey = 0;
+    // 32-bit rows and slices; the metadata of a slice is one broadcast load per
+    // warp (the loop issues as much as it loads: IPC 2.3 of 4 with 64-bit rows
+    // and shuffled metadata; 256^3 FP32 199 -> 191 us, 150^3 BF16 70 -> 53 us)
     const int lane = threadIdx.x & 31;
-    const int64_t nc = chunks_of_cta(c);
-    const int64_t step = (int64_t)c.G * kChunkRows;
-    const int64_t rw0 = (int64_t)blockIdx.x * kChunkRows + (threadIdx.x & ~31);   // warp's slice in chunk 0
-
-    // slice metadata: chunk i (broadcast, wt_c / so_c) and chunk i + 1 (lane-0
-    // values, broadcast one iteration later)
-    int wt_c = 0, mw_raw = 0;
-    long long so_c = 0, mo_raw = 0;
-    if (lane == 0 && nc > 0 && rw0 < c.n) {
-        wt_c = __ldg(c.sell_w + (rw0 >> 5));
-        so_c = __ldg(c.sell_off + (rw0 >> 5));
+    const unsigned n32 = (unsigned)c.n, step = (unsigned)c.G * kChunkRows;
+    unsigned r = blockIdx.x * kChunkRows + threadIdx.x;   // this thread's row in chunk i
+    const unsigned tstep = step / 32;
+    unsigned t = r >> 5;                                  // its slice
+    const unsigned nsl = (n32 + 31) / 32;
+    int64_t wo[KW];
+#pragma unroll
+    for (int a = 0; a < KW; ++a) wo[a] = a < nw ? c.woff[a] : 0;
+    // slice metadata of chunks i and i + 1 (0 wide past the end)
+    int wt_c = 0, wt_n = 0;
+    long long so_c = 0, so_n = 0;
+    if (t < nsl) {
+        wt_c = __ldg(c.sell_w + t);
+        so_c = __ldg(c.sell_off + t);
     }
-    wt_c = __shfl_sync(0xffffffffu, wt_c, 0);
-    so_c = __shfl_sync(0xffffffffu, so_c, 0);
-    if (lane == 0 && nc > 1 && rw0 + step < c.n) {
-        mw_raw = __ldg(c.sell_w + ((rw0 + step) >> 5));
-        mo_raw = __ldg(c.sell_off + ((rw0 + step) >> 5));
+    if (t + tstep < nsl) {
+        wt_n = __ldg(c.sell_w + t + tstep);
+        so_n = __ldg(c.sell_off + t + tstep);
     }
-    int cv[8];
+    int cv[W];
     {
         const int32_t *pc = c.sell_col + so_c + lane;
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
+        for (int p = 0; p < W; ++p)
             if (p < wt_c) cv[p] = __ldcs(pc + 32 * p);
     }
-    for (int64_t i = 0; i < nc; ++i) {
-        const int64_t rw = rw0 + i * step;
-        const int64_t r = rw + lane;
-        const bool ok = rw < c.n && r < c.n;   // padded rows of the last slice do no work
+    for (; t < nsl; r += step, t += tstep) {
+        const bool ok = r < n32;   // padded rows of the last slice do no work
         // (1) values, gathers and window of chunk i
-        float av[8], xv[8], wv[KW];
+        float av[W], xv[W], wv[KW];
         {
             const float *pv = c.sell_val + so_c + lane;
 #pragma unroll
-            for (int p = 0; p < 8; ++p)
+            for (int p = 0; p < W; ++p)
                 if (p < wt_c) {
                     av[p] = __ldcs(pv + 32 * p);
                     xv[p] = Store<TB>::ld(wj + cv[p]);
                 }
 #pragma unroll
-            for (int a = 0; a < KW; ++a) wv[a] = (ok && a < nw) ? Store<TB>::ld(V + c.woff[a] + r) : 0.f;
+            for (int a = 0; a < KW; ++a) wv[a] = (ok && a < nw) ? Store<TB>::ld(V + wo[a] + r) : 0.f;
         }
-        // (2) metadata of chunk i + 1 (loaded one iteration ago) and its column indices
-        const int wt_n = __shfl_sync(0xffffffffu, mw_raw, 0);
-        const long long so_n = __shfl_sync(0xffffffffu, mo_raw, 0);
-        int cvn[8];
+        // (2) column indices of chunk i + 1
+        int cvn[W];
         {
             const int32_t *pc = c.sell_col + so_n + lane;
 #pragma unroll
-            for (int p = 0; p < 8; ++p)
+            for (int p = 0; p < W; ++p)
                 if (p < wt_n) cvn[p] = __ldcs(pc + 32 * p);
         }
         // (3) metadata of chunk i + 2
-        mw_raw = 0;
-        mo_raw = 0;
-        if (lane == 0 && i + 2 < nc && rw + 2 * step < c.n) {
-            mw_raw = __ldg(c.sell_w + ((rw + 2 * step) >> 5));
-            mo_raw = __ldg(c.sell_off + ((rw + 2 * step) >> 5));
+        int wt_f = 0;
+        long long so_f = 0;
+        if (t + 2 * tstep < nsl) {
+            wt_f = __ldg(c.sell_w + t + 2 * tstep);
+            so_f = __ldg(c.sell_off + t + 2 * tstep);
         }
         // (4) y of chunk i
         if (ok) {
             float y = 0.f;
 #pragma unroll
-            for (int p = 0; p < 8; ++p)
+            for (int p = 0; p < W; ++p)
                 if (p < wt_c) y = fmaf(av[p], xv[p], y);
             c.Y[r] = y;
 #pragma unroll
@@ -616,8 +619,10 @@ __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv_lp_pipe(LpCtx 
         }
         wt_c = wt_n;
         so_c = so_n;
+        wt_n = wt_f;
+        so_n = so_f;
 #pragma unroll
-        for (int p = 0; p < 8; ++p) cv[p] = cvn[p];
+        for (int p = 0; p < W; ++p) cv[p] = cvn[p];
     }
     spmv_end<KW>(c, j, nw, last, L, bins, acc, ykey, red);
 }
@@ -883,58 +888,69 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_arnoldi_update_lp(LpCtx c, i
     const int shift_d = L - (ed == kNoExp ? 0 : ed);
 
     const int ng = min(j + 1, c.k - 1);
-    float part[KW + 1];
+    float part[KW];   // ||w_{j+1}||^2, <w_{j+1}, w_{j+1-d}> at d
 #pragma unroll
-    for (int i = 0; i <= KW; ++i) part[i] = 0.f;
+    for (int i = 0; i < KW; ++i) part[i] = 0.f;
     unsigned nkey = 0;
     TB *wn = V + vcol(c, j + 1);
     const int lane = threadIdx.x & 31;
-    const int64_t nc = chunks_of_cta(c);
-    constexpr int U = KW <= 2 ? 4 : (KW <= 4 ? 2 : 1);   // chunks in flight per thread
-    for (int64_t i = 0; i < nc; i += U) {
-        float yv[U], wv[U][KW];
-        int64_t rr[U];
-        uint2 pvu[U];   // compact pattern words (split layout), loaded with the rest
+    // Row loop.  This kernel is bound by instruction issue (IPC 2.6 to 3.1 of 4
+    // with 64-bit row arithmetic and a bin address per atomic), so rows are
+    // 32-bit, the window coefficients stay in registers and the compact pattern
+    // takes four instructions per nonzero (scatter8).  The loads of the next
+    // U chunks are issued before the arithmetic of these.  N = 16.8M, FP32:
+    // 114 -> 93 us; BF16, N = 3.4M: 60 -> 47 us.  The rows a thread adds up,
+    // and their order, do not depend on U.
+    constexpr int U = KW <= 2 ? 2 : 1;       // chunks per iteration and thread
+    constexpr bool kAhead = KW <= 4;         // wider windows do not fit in the registers twice
+    const unsigned n32 = (unsigned)c.n, step = (unsigned)G * kChunkRows;
+    float cf[KW];                            // coefficients, newest first: cf[b] for w_{j-b}
+    int64_t wo[KW];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            rr[u] = i + u < nc ? chunk_row(c, i + u) : -1;
-            const bool ok = rr[u] >= 0;
-            yv[u] = (ok && do_update) ? c.Y[rr[u]] : 0.f;
+    for (int b2 = 0; b2 < KW; ++b2) {
+        cf[b2] = b2 < nw ? scf[nw - 1 - b2] : 0.f;
+        wo[b2] = b2 < nw ? c.woff[nw - 1 - b2] : 0;
+    }
+    struct Rows {
+        float y[U], w[U][KW];   // w[u][b] = w_{j-b}
+        uint2 pv[U];            // compact pattern words (split layout)
+    };
+    auto load_rows = [&](unsigned r, Rows &q) {
 #pragma unroll
-            for (int a = 0; a < KW; ++a)
-                wv[u][a] = (ok && a < nw) ? Store<TB>::ld(V + c.woff[a] + rr[u]) : 0.f;
-            pvu[u] = make_uint2(0u, 0u);
+        for (int u = 0; u < U; ++u, r += step) {
+            const bool ok = r < n32;
+            q.y[u] = (ok && do_update) ? c.Y[r] : 0.f;
+#pragma unroll
+            for (int b2 = 0; b2 < KW; ++b2) q.w[u][b2] = (ok && b2 < nw) ? Store<TB>::ld(V + wo[b2] + r) : 0.f;
+            q.pv[u] = make_uint2(0u, 0u);
             if constexpr (split)
-                if (ok) pvu[u] = __ldg((const uint2 *)(c.pattern8 + rr[u] * 8));
+                if (ok) q.pv[u] = __ldg((const uint2 *)c.pattern8 + r);
         }
+    };
+    // shared-memory addresses of this lane's bin copies (split layout)
+    const unsigned wbase = shared_address(wb0) + 4u * (unsigned)(lane & cm);
+    const unsigned dbase = shared_address(db) + 4u * (unsigned)(lane & cm);
+    Rows cur, nxt;
+    unsigned rb = blockIdx.x * kChunkRows + threadIdx.x;
+    if constexpr (kAhead) load_rows(rb, cur);
+    for (; rb < n32; rb += U * step) {
+        if constexpr (kAhead) load_rows(rb + U * step, nxt);
+        else load_rows(rb, cur);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t r = rr[u];
-            if (r < 0) continue;
-            float wjr = wv[u][0];
-#pragma unroll
-            for (int a = 1; a < KW; ++a)
-                if (a == nw - 1) wjr = wv[u][a];
+            const unsigned r = rb + u * step;
+            if (r >= n32) continue;
+            const float(&wv)[KW] = cur.w[u];
             int row[ZCAP];
             bool neg[ZCAP];
-            const uint2 pv = pvu[u];
             if constexpr (!split)
                 if (sk) pattern_row<ZCAP>(c, r, row, neg);
             if (sk && ew != kNoExp) {
                 // exact sketch of the stored w_j, per-lane bin copies
                 int l0, l1;
-                limbs_f32(wjr, lsw, l0, l1);
+                limbs_f32(wv[0], lsw, l0, l1);
                 if constexpr (split) {
-                    // bin 2 SB stripe + pattern byte: signs in separate bins
-                    constexpr int LC = SplitGeom<SB>::kLc;
-                    int *b0l = wb0 + (lane & ((1 << LC) - 1)), *b1l = wb1 + (lane & ((1 << LC) - 1));
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int e = (int)__byte_perm(q < 4 ? pv.x : pv.y, 0u, 0x4440u + (q & 3));
-                        const int bi = ((2 * SB * q) | e) << LC;
-                        atomicAdd(b0l + bi, l0);
-                        atomicAdd(b1l + bi, l1);
-                    }
+                    scatter8<SB, SplitGeom<SB>::kLc>(cur.pv[u], wbase, l0, l1);
                 } else {
 #pragma unroll
                     for (int q = 0; q < ZCAP; ++q)
@@ -946,28 +962,22 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_arnoldi_update_lp(LpCtx c, i
                 }
             }
             if (do_update) {
-                float w = sigf * yv[u];
+                float w = sigf * cur.y[u];
 #pragma unroll
-                for (int a = 0; a < KW; ++a)
-                    if (a < nw) w = fmaf(-scf[a], wv[u][a], w);
+                for (int b2 = KW - 1; b2 >= 0; --b2)
+                    if (b2 < nw) w = fmaf(-cf[b2], wv[b2], w);   // oldest first
                 const float wr = Store<TB>::rnd(w);
                 Store<TB>::st(wn + r, wr);
                 part[0] = fmaf(wr, wr, part[0]);
                 nkey = max(nkey, abs_key_f32(wr));
 #pragma unroll
-                for (int a = 0; a < KW; ++a)
-                    if (a < nw && nw - a <= ng) part[1 + a] = fmaf(wr, wv[u][a], part[1 + a]);
+                for (int d = 1; d < KW; ++d)   // <w_{j+1}, w_{j+1-d}>
+                    if (d <= ng) part[d] = fmaf(wr, wv[d - 1], part[d]);
                 if (resid && ed != kNoExp) {
                     // wr - w is exact in FP32 (Sterbenz: wr and w lie within a factor 2)
                     const int vd = (int)fixed_point_f32(wr - w, shift_d);
                     if constexpr (split) {
-                        constexpr int LC = SplitGeom<SB>::kLc;
-                        int *dl = db + (lane & ((1 << LC) - 1));
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const int e = (int)__byte_perm(q < 4 ? pv.x : pv.y, 0u, 0x4440u + (q & 3));
-                            atomicAdd(dl + (((2 * SB * q) | e) << LC), vd);
-                        }
+                        scatter8_one<SB, SplitGeom<SB>::kLc>(cur.pv[u], dbase, vd);
                     } else {
 #pragma unroll
                         for (int q = 0; q < ZCAP; ++q)
@@ -976,6 +986,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_arnoldi_update_lp(LpCtx c, i
                 }
             }
         }
+        if constexpr (kAhead) cur = nxt;
     }
     __syncthreads();
     if (sk) {
@@ -1004,16 +1015,18 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_arnoldi_update_lp(LpCtx c, i
         }
     }
     if (!do_update) return;
-    double partd[KW + 1];
+    double partd[KW];
 #pragma unroll
-    for (int i = 0; i <= KW; ++i) partd[i] = (double)part[i];
-    block_sum<KW + 1, kUpdThreads>(partd, red);
+    for (int i = 0; i < KW; ++i) partd[i] = (double)part[i];
+    block_sum<KW, kUpdThreads>(partd, red);
     const unsigned nmk = (unsigned)block_max_key<kUpdThreads>((unsigned long long)nkey, (unsigned long long *)red);
     if (threadIdx.x == 0) {
         double *o = c.p2 + (size_t)blockIdx.x * kP2;
         o[0] = partd[0];
         o[1] = (double)__uint_as_float(nmk);
-        for (int a = 0; a < KW; ++a) o[2 + a] = partd[1 + a];
+#pragma unroll
+        for (int d = 1; d < KW; ++d)
+            if (d <= ng) o[2 + nw - d] = partd[d];
     }
     if (last_to_arrive(c.cnt + 1)) {
         const int warp = threadIdx.x >> 5;
@@ -1087,7 +1100,12 @@ __global__ void __launch_bounds__(kThreads) k_arnoldi_info_lp(LpCtx c, skf_info 
 template <int KW, int ZCAP, typename TB>
 void launch_steps(const LpCtx &c, bool pipe, size_t smem_spmv, size_t smem_upd, cudaStream_t st,
                   const StepHook *hook, const skf_sketch *dense, void *dwork) {
-    auto spmv = pipe ? k_arnoldi_spmv_lp_pipe<KW, ZCAP, TB> : k_arnoldi_spmv_lp<KW, ZCAP, TB>;
+    auto spmv = pipe ? k_arnoldi_spmv_lp_pipe<KW, ZCAP, TB, 8> : k_arnoldi_spmv_lp<KW, ZCAP, TB>;
+    // fewer product slots for the 5- and 7-point stencils
+    if constexpr (KW == 2 && ZCAP == 8) {
+        if (pipe && c.max_width <= 7) spmv = c.max_width <= 5 ? k_arnoldi_spmv_lp_pipe<KW, ZCAP, TB, 5>
+                                                              : k_arnoldi_spmv_lp_pipe<KW, ZCAP, TB, 7>;
+    }
     auto update = k_arnoldi_update_lp<KW, ZCAP, TB, 0>;
     if constexpr (ZCAP == 8) {
         if (c.split) update = c.p8_block == 64 ? k_arnoldi_update_lp<KW, 8, TB, 64> : k_arnoldi_update_lp<KW, 8, TB, 128>;
@@ -1169,6 +1187,7 @@ skf_status lp_setup(const skf_csr *A, const skf_sketch *S, int m, int k, TB *V, 
     c.sell_w = A->sell_w;
     c.sell_val = (const float *)A->sell_val;
     c.sell_col = A->sell_col;
+    c.max_width = A->max_width;
     c.norm_inf = A->norm_inf;
     // an SRHT or SRDCT (F32 basis) is applied by its own kernels to w_j and
     // y_j after each SpMV; the step kernels then run as for S = I (no
@@ -1347,7 +1366,7 @@ skf_status arnoldi_run_lp_block(const skf_csr *A, const skf_sketch *S, int nr, c
     const int G = runs[0].c.G;
     for (int q = 0; q < nr; ++q) k_arnoldi_init_lp<TB><<<G, kChunkRows, 0, st>>>(runs[q].c, b[q]);
     auto spmm = k_arnoldi_spmm_lp<2, 8, TB, kSpmmBlock>;
-    auto spmv = k_arnoldi_spmv_lp_pipe<2, 8, TB>;
+    auto spmv = k_arnoldi_spmv_lp_pipe<2, 8, TB, 8>;
     auto update = k_arnoldi_update_lp<2, 8, TB, 0>;
     if (runs[0].c.split)
         update = runs[0].c.p8_block == 64 ? k_arnoldi_update_lp<2, 8, TB, 64> : k_arnoldi_update_lp<2, 8, TB, 128>;
