@@ -620,6 +620,7 @@ static skf_status solve_enqueue(skf_method method, const skf_csr *A, const skf_s
         sc.stop_tol = p.stop_tol;
         sc.err = SKF_OK;
         hook.fn = stop_hook;
+        hook.every = p.check_every;
         hook.ctx = &sc;
     }
     double *z = nullptr;

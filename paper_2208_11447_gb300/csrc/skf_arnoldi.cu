@@ -7,14 +7,27 @@
 //
 //   spmv   (step j): y~ = A w_j on the CTA's rows -> Y; partial dots
 //                    <w_i, y~> (i in the window) and max|y~|; in its
-//                    prologue, S v_{j-1} and S A v_{j-1} from the update's
-//                    integer partials.
+//                    prologue, S v_{j-1} from the update's integer partials,
+//                    and S A v_{j-2}.
 //   update (step j): MGS coefficients from the reduced dots and the window
 //                    Gram matrix (identical to MGS in exact arithmetic),
 //                    w_{j+1} = sigma_j y~ - sum_i h_ij sigma_i w_i, partial
 //                    ||w_{j+1}||^2, max|w_{j+1}| and the Gram entries
-//                    <w_{j+1}, w_i> of the next window; fixed-point sketches
-//                    of w_j (-> S v_j) and of y~ (-> S A v_j).
+//                    <w_{j+1}, w_i> of the next window; fixed-point sketch
+//                    of w_j (-> S v_j).
+//
+// S A v_j is not sketched row by row.  The update of step j applied
+// w_{j+1} = sigma_j y~ - sum_i c_i w_i, so S A v_j = sigma_j S y~ = S w_{j+1} +
+// sum_i c_i S w_i, the sketched Arnoldi relation with the very coefficients
+// the update used: it differs from a direct sketch by the sketch of the
+// update's own rounding (about one unit roundoff of ||A v_j||), as in the
+// persistent form.  Only the last S y~ (and with the stopping criterion those of
+// the steps before a checkpoint, so that a checkpoint sees what a run of that
+// length sees) is sketched directly; at a happy breakdown the noise vector w_{m_eff} is sketched once more to close the last
+// relation.  One sketched vector per step instead of two, the update's shared
+// atomics (16 per row and vector) and the SRDCT's transforms halved:
+// N = 4.0e6, zeta = 8: update 77 -> 66 us; SRDCT at N = 3.6e5: one transform
+// per step instead of two.
 //
 // Cross-CTA reductions: every CTA writes its partials; the CTA that arrives
 // last (atomic ticket, no waiting) reduces them in a fixed order and publishes
@@ -54,6 +67,7 @@ struct ArnCtx {
     int srht_frac;     // SRHT fixed-point fraction bits
     double sk_scale;   // scale of the integer sums: 1/sqrt(zeta) or 1/sqrt(s)
     int m, k;
+    int every;         // > 0: checkpoints of the stopping criterion at every, 2 every, ... columns
     double *V;
     int64_t ldv;
     int vring;         // 0: V holds all m columns; > 0: a ring of vring slots (two-pass)
@@ -70,7 +84,9 @@ struct ArnCtx {
     double inv_sqrt_zeta;
     unsigned *cnt;     // [2] arrival tickets of the spmv / update launches
     long long *skSV;   // [G][s]
-    long long *skSAV;  // [G][s]
+    long long *skSAV;  // [G][s] S y~_{m-1}
+    double *Sw;        // [m + 1][s] S w_j (unnormalised)
+    double *coef;      // [m][kMaxK] coefficients of update j, newest first: coef[b] for w_{j-b}
     double *gram;      // [m][kMaxK]: <w_j, w_{j-d}>, d = 1..k-1 (reduced by the update kernel of step j-1)
     int *eys;          // [m] exponent of max|y~_j| (kNoExp if zero)
     int *ews;          // [m] exponent of max|w_j|
@@ -85,18 +101,43 @@ struct ArnCtx {
 
 namespace {
 
-// Finalise a sketch column from the integer partials, for this CTA's slice of
-// the s rows: one warp per row of S.
-__device__ __forceinline__ void finalize_sketch(const long long *part, int G, int s, int E, int frac, double scale,
-                                                double *out_col) {
+// S y~_j is sketched directly (else by the relation).
+__host__ __device__ __forceinline__ bool y_direct(const ArnCtx &c, int j) {
+    return j == c.m - 1 || (c.every > 0 && j >= 0 && (j + 1) % c.every == 0);
+}
+
+// Row i of a sketch column from the integer partials, by one warp.
+__device__ __forceinline__ double sketch_row(const long long *part, int G, int s, int i, int E, int frac, double scale) {
+    return E != kNoExp ? scale_pow2(warp_sum_i64_exact(part + i, G, (size_t)s), E - frac) * scale : 0.0;
+}
+
+// S w_jw from the partials of its step (an SRDCT has written it) for this
+// CTA's slice of the rows of S; then S A v_{jw-1} by the relation (see above)
+// unless it is sketched directly; with `store` (jw < m_eff) S v_jw and, where
+// y~_jw is sketched directly, S A v_jw from its partials.
+__device__ __forceinline__ void finalize_column(const ArnCtx &c, int jw, bool store) {
+    const bool rel = jw >= 1 && !y_direct(c, jw - 1), ydir = store && !c.direct && y_direct(c, jw);
+    const int s = c.sp.s;
     const int per = (s + gridDim.x - 1) / gridDim.x;
-    const int i0 = blockIdx.x * per;
-    const int i1 = min(s, i0 + per);
+    const int b0 = blockIdx.x * per, b1 = min(s, b0 + per);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = i0 + warp; i < i1; i += blockDim.x / 32) {
-        double v = 0.0;
-        if (E != kNoExp) v = scale_pow2(warp_sum_i64_exact(part + i, G, (size_t)s), E - frac) * scale;
-        if (lane == 0) out_col[i] = v;
+    const int frac = c.direct ? 0 : c.srht ? c.srht_frac : sketch_fraction_bits_from_limb(limb_bits(*c.binmax));
+    const int nw = jw >= 1 ? min(jw, c.k) : 0;   // window length of step jw - 1
+    const double *cf = c.coef + (size_t)max(jw - 1, 0) * kMaxK;
+    for (int i = b0 + warp; i < b1; i += blockDim.x / 32) {
+        const double sw = c.direct ? __ldcg(c.Sw + (size_t)jw * s + i)
+                                   : sketch_row(c.skSV, c.sk_parts, s, i, c.ews[jw], frac, c.sk_scale);
+        const double sy = ydir ? sketch_row(c.skSAV, c.sk_parts, s, i, c.eys[jw], frac, c.sk_scale) : 0.0;
+        if (lane == 0) {
+            if (!c.direct) c.Sw[(size_t)jw * s + i] = sw;
+            if (store) c.SV[i + (size_t)jw * s] = c.vscale[jw] * sw;
+            if (rel) {
+                double v = sw;
+                for (int b = nw - 1; b >= 0; --b) v = fma(cf[b], c.Sw[(size_t)(jw - 1 - b) * s + i], v);
+                c.SAV[i + (size_t)(jw - 1) * s] = v;
+            }
+            if (ydir) c.SAV[i + (size_t)jw * s] = c.vscale[jw] * sy;
+        }
     }
 }
 
@@ -171,15 +212,9 @@ __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv(ArnCtx c, int 
     // recomputed identically by every CTA below
     if (c.iscal[0] && c.iscal[3] < j) return;
     const int G = gridDim.x;
-    const int s = c.sp.s;
 
-    // S v_{j-1} and S A v_{j-1} from the integer partials of the previous step
-    if (j >= 1 && !c.identity && !c.direct) {
-        const int frac = c.srht ? c.srht_frac : sketch_fraction_bits_from_limb(limb_bits(*c.binmax));
-        const double sc = c.vscale[j - 1] * c.sk_scale;
-        finalize_sketch(c.skSV, c.sk_parts, s, c.ews[j - 1], frac, sc, c.SV + (size_t)(j - 1) * s);
-        finalize_sketch(c.skSAV, c.sk_parts, s, c.eys[j - 1], frac, sc, c.SAV + (size_t)(j - 1) * s);
-    }
+    // S v_{j-1} from the integer partials of the previous step, S A v_{j-2}
+    if (j >= 1 && !c.identity) finalize_column(c, j - 1, true);
 
     // zero right-hand side (j = 0) or happy breakdown ||w_j|| <= 1e-12 ||A v_{j-1}||,
     // decided once by the previous launch
@@ -287,10 +322,13 @@ __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv(ArnCtx c, int 
 // k_arnoldi_spmv.
 constexpr int kPipeRows = 512;
 
-// CTAs of the pipelined SpMV: one per SM, at most one per chunk.
-inline int pipe_ctas(int64_t n) {
+// CTAs of the pipelined SpMV: one per SM, at most one per chunk or per
+// kFinRows rows of S, of which its prologue finalises a column (few chunks and
+// many rows left several rows to each warp: N = 4096, s = 640: 18.8 -> 11.6 us).
+constexpr int kFinRows = 16;
+inline int pipe_ctas(int64_t n, int s) {
     const int64_t chunks = (n + kPipeRows - 1) / kPipeRows;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(chunks, num_sms()));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::max<int64_t>(chunks, s / kFinRows), num_sms()));
 }
 
 template <int KW, int W>
@@ -303,13 +341,7 @@ __global__ void __launch_bounds__(kPipeRows, 1) k_arnoldi_spmv_pipe(ArnCtx c, in
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (c.iscal[0] && c.iscal[3] < j) return;
     const int G = gridDim.x;
-    const int s = c.sp.s;
-    if (j >= 1 && !c.identity && !c.direct) {
-        const int frac = c.srht ? c.srht_frac : sketch_fraction_bits_from_limb(limb_bits(*c.binmax));
-        const double sc = c.vscale[j - 1] * c.sk_scale;
-        finalize_sketch(c.skSV, c.sk_parts, s, c.ews[j - 1], frac, sc, c.SV + (size_t)(j - 1) * s);
-        finalize_sketch(c.skSAV, c.sk_parts, s, c.eys[j - 1], frac, sc, c.SAV + (size_t)(j - 1) * s);
-    }
+    if (j >= 1 && !c.identity) finalize_column(c, j - 1, true);
     const double *sc_j = c.stepsc + 4 * (size_t)j;
     if (j >= 1 && blockIdx.x == 0 && threadIdx.x == 0) c.H[j + (size_t)(j - 1) * (c.m + 1)] = sc_j[1];
     if (sc_j[2] != 0.0) {
@@ -486,7 +518,10 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     // programmatic dependent of the SpMV launch (see k_arnoldi_spmv_pipe)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (c.iscal[0] && c.iscal[3] <= j) return;   // stopped at this step (set by its spmv launch) or earlier
+    // stopped at this step (set by its SpMV launch) or earlier; at a happy
+    // breakdown at this step only w_j is sketched
+    const bool stop_here = c.iscal[0] == 1 && c.iscal[3] == j && j >= 1;
+    if (c.iscal[0] && c.iscal[3] <= j && (!stop_here || c.identity)) return;
     const int G = gridDim.x;
     const double *fd = c.fin_d + (size_t)j * kP1;
     const double sigma = c.stepsc[4 * (size_t)j];
@@ -496,7 +531,7 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     const int i0 = max(0, j - c.k + 1);
     const int nw = j - i0 + 1;
 
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && !stop_here) {
         // MGS in the window, ascending, from the dots and the Gram matrix:
         // h_i = <v_i, y> - sum_{i' < i} h_i' <v_i, v_i'>.
         for (int a = 0; a < nw; ++a) {
@@ -515,16 +550,24 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     }
     __syncthreads();
     const int ey = positive_finite(ymax) ? bound_exponent(ymax) : kNoExp;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0 && !stop_here) {
         c.vscale[j] = sigma;
         c.eys[j] = ey;
+        for (int a = 0; a < nw; ++a) c.coef[(size_t)j * kMaxK + a] = scoef[a];
         if (j < c.m - 1)
             for (int a = 0; a < nw; ++a) c.H[(i0 + a) + (size_t)j * (c.m + 1)] = sh[a];
     }
-    // fixed-point sketches of w_j (-> S v_j) and y~ (-> S A v_j), two limbs each
-    int *aw0 = bins, *aw1 = bins + s, *ay0 = bins + 2 * s, *ay1 = bins + 3 * s;
+    // fixed-point sketch of w_j (-> S v_j) and, where it is not formed by the
+    // relation, of y~ (-> S A v_j), two limbs each.  Compact pattern: bins laid out
+    // [stripe][sign][p8_block], so that a pattern byte is a bin offset and no
+    // sign has to be applied.
+    const bool do_update = j < c.m - 1 && !stop_here;
+    const bool ylast = c.sparse && y_direct(c, j) && !stop_here;
+    const bool p8 = ZCAP == 8 && c.sparse && c.pattern8 != nullptr;
+    const int nbin = p8 ? 16 * c.p8_block : s;
+    int *aw0 = bins, *aw1 = bins + nbin, *ay0 = bins + 2 * nbin, *ay1 = bins + 3 * nbin;
     if (c.sparse)
-        for (int i = threadIdx.x; i < 4 * s; i += kUpdThreads) bins[i] = 0;
+        for (int i = threadIdx.x; i < (ylast ? 4 : 2) * nbin; i += kUpdThreads) bins[i] = 0;
     __syncthreads();
     const int L = c.sparse ? limb_bits(*c.binmax) : 0;
     const int frac = sketch_fraction_bits_from_limb(L);
@@ -533,7 +576,6 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     if (blockIdx.x == 0 && threadIdx.x == 0) c.ews[j] = ew;
     const int shift_w = frac - (ew == kNoExp ? 0 : ew);
     const int shift_y = frac - (ey == kNoExp ? 0 : ey);
-    const bool do_update = j < c.m - 1;
     // part[0] = ||w_{j+1}||^2, part[d] = <w_{j+1}, w_{j+1-d}> for the Gram
     // distances d = 1 .. ng of the next window (ng <= KW - 1): only the live
     // products are issued (a predicated-off DFMA still takes FP64 pipe time)
@@ -549,59 +591,75 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     int64_t woffr[KW];
 #pragma unroll
     for (int b = 0; b < KW; ++b) woffr[b] = b < nw ? c.woff[nw - 1 - b] : 0;
-    // four rows per thread per iteration, all loads (with the compact sketch
-    // pattern, where there is one) issued before the arithmetic
-    constexpr int U = 4;
-    const bool p8 = ZCAP == 8 && c.sparse && c.pattern8 != nullptr;
-    for (int64_t rb = r0 + threadIdx.x; rb < r1; rb += U * kUpdThreads) {
-        double yv[U], wv[U][KW];   // wv[u][b] = w_{j-b}: newest first
-        uint2 pvu[U];
+    // Two rows per thread and iteration; the loads of the next two (with their
+    // compact sketch patterns) are issued before the arithmetic of these.
+    constexpr int U = 2;
+    const int rn = (int)(r1 - r0);   // rows of this CTA (32-bit offsets from here on)
+    const double *Yc = c.Y + r0;
+    const double *Vc = c.V + r0;
+    const uint8_t *p8c = p8 ? c.pattern8 + r0 * 8 : nullptr;
+    wn += r0;
+    const unsigned wbase = shared_address(aw0), ybase = shared_address(ay0);
+    double cf[KW];
+#pragma unroll
+    for (int a = 0; a < KW; ++a) cf[a] = a < nw ? scoef[a] : 0.0;
+    struct Rows {
+        double y[U], w[U][KW];   // w[u][b] = w_{j-b}: newest first
+        uint2 pv[U];
+    };
+    auto load_rows = [&](int x, Rows &q) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t r = rb + (int64_t)u * kUpdThreads;
-            const bool ok = r < r1;
-            yv[u] = ok ? c.Y[r] : 0.0;
+            const int xr = x + u * kUpdThreads;
+            const bool ok = xr < rn;
+            q.y[u] = ok ? Yc[xr] : 0.0;
 #pragma unroll
-            for (int a = 0; a < KW; ++a)
-                wv[u][a] = (ok && a < nw) ? c.V[r + woffr[a]] : 0.0;
-            pvu[u] = (ok && p8) ? __ldg((const uint2 *)(c.pattern8 + r * 8)) : make_uint2(0u, 0u);
+            for (int a = 0; a < KW; ++a) q.w[u][a] = (ok && a < nw) ? Vc[xr + woffr[a]] : 0.0;
+            q.pv[u] = (ok && p8) ? __ldg((const uint2 *)p8c + xr) : make_uint2(0u, 0u);
         }
+    };
+    constexpr bool kPrefetch = KW <= 2;   // wider windows do not fit in the registers twice
+    Rows cur, nxt;
+    if constexpr (kPrefetch) load_rows(threadIdx.x, cur);
+    for (int x = threadIdx.x; x < rn; x += U * kUpdThreads) {
+        if constexpr (kPrefetch) load_rows(x + U * kUpdThreads, nxt);
+        else load_rows(x, cur);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t r = rb + (int64_t)u * kUpdThreads;
-            if (r < r1) {
-                const double y = yv[u];
-                const double wjr = wv[u][0];
+            const int xr = x + u * kUpdThreads;
+            if (xr < rn) {
+                const int64_t r = r0 + xr;
+                const double y = cur.y[u];
+                const double wjr = cur.w[u][0];
                 if (do_update) {
                     double w = sigma * y;
 #pragma unroll
                     for (int a = 0; a < KW; ++a)
-                        if (KW - 1 - a < nw) w = fma(-scoef[KW - 1 - a], wv[u][KW - 1 - a], w);   // oldest first
-                    wn[r] = w;
+                        if (KW - 1 - a < nw) w = fma(-cf[KW - 1 - a], cur.w[u][KW - 1 - a], w);   // oldest first
+                    wn[xr] = w;
                     part[0] = fma(w, w, part[0]);
                     nkey = max(nkey, abs_key(w));
 #pragma unroll
                     for (int d = 1; d < KW; ++d) {
-                        if (d <= ng) part[d] = fma(w, wv[u][d - 1], part[d]);   // w_{j+1-d}
+                        if (d <= ng) part[d] = fma(w, cur.w[u][d - 1], part[d]);   // w_{j+1-d}
                     }
                 }
                 if (c.identity) {
                     c.SV[r + (size_t)j * s] = sigma * wjr;
                     c.SAV[r + (size_t)j * s] = sigma * y;
                 } else if (c.sparse) {
-                    const long long vw = fixed_point(wjr, shift_w);
-                    const long long vy = ey == kNoExp ? 0 : fixed_point(y, shift_y);
+                    const long long vw = ew == kNoExp ? 0 : fixed_point(wjr, shift_w);
+                    const long long vy = (!ylast || ey == kNoExp) ? 0 : fixed_point(y, shift_y);
                     const int w0 = (int)(vw & lmask), w1 = (int)(vw >> L);
                     const int y0 = (int)(vy & lmask), y1 = (int)(vy >> L);
                     if (p8) {
-                        const uint2 pv = pvu[u];
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const int e = (int)__byte_perm(q < 4 ? pv.x : pv.y, 0u, 0x4440u + (q & 3));
-                            const bool neg = e >= c.p8_block;
-                            const int row = c.sp.start[q] + (neg ? e - c.p8_block : e);
-                            red_limbs(aw0, aw1, row, w0, w1, neg);
-                            red_limbs(ay0, ay1, row, y0, y1, neg);
+                        const uint2 pv = cur.pv[u];
+                        if (c.p8_block == 64) {
+                            scatter8<64, 0>(pv, wbase, w0, w1);
+                            if (ylast) scatter8<64, 0>(pv, ybase, y0, y1);
+                        } else {
+                            scatter8<128, 0>(pv, wbase, w0, w1);
+                            if (ylast) scatter8<128, 0>(pv, ybase, y0, y1);
                         }
                     } else {
                         uint16_t e[ZCAP];
@@ -613,14 +671,36 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
                                 bool neg;
                                 pattern_entry(c.sp, e[q], q, row, neg);
                                 red_limbs(aw0, aw1, row, w0, w1, neg);
-                                red_limbs(ay0, ay1, row, y0, y1, neg);
+                                if (ylast) red_limbs(ay0, ay1, row, y0, y1, neg);
                             }
                         }
                     }
                 }
             }
         }
+        if constexpr (kPrefetch) cur = nxt;
     }
+    if (c.sparse) {
+        __syncthreads();
+        long long *ow = c.skSV + (size_t)blockIdx.x * s, *oy = c.skSAV + (size_t)blockIdx.x * s;
+        if (p8) {
+            const int blk = c.p8_block, lb = blk == 64 ? 6 : 7;
+            for (int x = threadIdx.x; x < 8 * blk; x += kUpdThreads) {
+                const int q = x >> lb, i = x & (blk - 1);
+                if (i < c.sp.size[q]) {
+                    const int row = c.sp.start[q] + i, o = x + q * blk;
+                    ow[row] = combine_limbs(aw0[o] - aw0[o + blk], aw1[o] - aw1[o + blk], L);
+                    if (ylast) oy[row] = combine_limbs(ay0[o] - ay0[o + blk], ay1[o] - ay1[o + blk], L);
+                }
+            }
+        } else {
+            for (int i = threadIdx.x; i < s; i += kUpdThreads) {
+                ow[i] = combine_limbs(aw0[i], aw1[i], L);
+                if (ylast) oy[i] = combine_limbs(ay0[i], ay1[i], L);
+            }
+        }
+    }
+    if (stop_here) return;
     block_sum_auto<KW, kUpdThreads>(part, red);
     const double nmax = key_to_abs(block_max_key<kUpdThreads>(nkey, (unsigned long long *)red));
     if (threadIdx.x == 0) {
@@ -631,14 +711,6 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
 #pragma unroll
         for (int d = 1; d < KW; ++d)
             if (d <= ng) o[2 + nw - d] = part[d];
-    }
-    if (c.sparse) {
-        __syncthreads();
-        long long *ow = c.skSV + (size_t)blockIdx.x * s, *oy = c.skSAV + (size_t)blockIdx.x * s;
-        for (int i = threadIdx.x; i < s; i += kUpdThreads) {
-            ow[i] = combine_limbs(aw0[i], aw1[i], L);
-            oy[i] = combine_limbs(ay0[i], ay1[i], L);
-        }
     }
     if (last_to_arrive(c.cnt + 1)) {
         const int warp = threadIdx.x >> 5;
@@ -670,14 +742,14 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     }
 }
 
-// After the loop: S v_{m-1} and S A v_{m-1}.
+// After the loop: the pending columns.  Ran to the end: S v_{m-1}, S A v_{m-2}
+// by the relation and the sketched S A v_{m-1}.  Happy breakdown at step me:
+// S w_me (not a basis column) gives S A v_{me-1}.
 __global__ void __launch_bounds__(kThreads) k_arnoldi_finish(ArnCtx c) {
-    if (c.iscal[0] == 0 && !c.identity && !c.direct) {
-        const int frac = c.srht ? c.srht_frac : sketch_fraction_bits_from_limb(limb_bits(*c.binmax));
-        const double sc = c.vscale[c.m - 1] * c.sk_scale;
-        finalize_sketch(c.skSV, c.sk_parts, c.sp.s, c.ews[c.m - 1], frac, sc, c.SV + (size_t)(c.m - 1) * c.sp.s);
-        finalize_sketch(c.skSAV, c.sk_parts, c.sp.s, c.eys[c.m - 1], frac, sc, c.SAV + (size_t)(c.m - 1) * c.sp.s);
-    }
+    const int me = c.iscal[1];
+    if (me == 0 || c.identity || c.iscal[0] == 2) return;   // (2: stopped by the criterion, columns < me are final)
+    if (c.iscal[0] != 0) finalize_column(c, me, false);
+    else finalize_column(c, c.m - 1, true);
 }
 
 // | ||S v_j||^2 - 1 | per column (the embedding-quality estimate of Sec. 4.3),
@@ -722,9 +794,11 @@ void launch_steps(const ArnCtx &c, int G, int Gs, size_t smem, const SrhtDev *sd
     // or 8 (a slot past a slice's width is a predicated-off FP64 instruction)
     auto spmv_pipe = c.max_width <= 5 ? k_arnoldi_spmv_pipe<KW, 5>
                    : c.max_width <= 7 ? k_arnoldi_spmv_pipe<KW, 7> : k_arnoldi_spmv_pipe<KW, 8>;
-    const int Gp = pipe_ctas(c.n);
+    const int Gp = pipe_ctas(c.n, c.identity ? 0 : c.sp.s);
     auto update = k_arnoldi_update<KW, ZCAP>;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (beside up to 33 KB of static shared memory)
+    if (2 * smem > 12 * 1024)
+        cudaFuncSetAttribute(update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * smem));
     // the pipelined SpMV and the update are launched as programmatic
     // dependents of the launch before them (each waits for it in full)
     cudaLaunchAttribute pdl[1];
@@ -738,7 +812,6 @@ void launch_steps(const ArnCtx &c, int G, int Gs, size_t smem, const SrhtDev *sd
     cfg_s.numAttrs = 1;
     cfg_u.gridDim = dim3((unsigned)G);
     cfg_u.blockDim = dim3(kUpdThreads);
-    cfg_u.dynamicSmemBytes = smem;
     cfg_u.stream = st;
     cfg_u.attrs = pdl;
     cfg_u.numAttrs = 1;
@@ -748,32 +821,38 @@ void launch_steps(const ArnCtx &c, int G, int Gs, size_t smem, const SrhtDev *sd
         if (c.rs.sell_long) k_spmv_long<<<long_ctas(c.rs.nseg, num_sms()), 256, 0, st>>>(cj, j);
         if (pipe) cudaLaunchKernelEx(&cfg_s, spmv_pipe, cj, j);
         else spmv<<<Gs, kSpmvThreads, 0, st>>>(cj, j);
-        call_hook(hook, j, st);   // S v_i, S A v_i final for i < j
+        // S v_i, S A v_i final for i < j at a checkpoint (S A v_{j-1} sketched directly), else i < j - 1
+        if (y_direct(c, j - 1)) call_hook(hook, j, st);
+        const bool ydir = y_direct(c, j);
+        cfg_u.dynamicSmemBytes = ydir ? 2 * smem : smem;
         cudaLaunchKernelEx(&cfg_u, update, cj, j);
         if (j + 1 < c.m) call_col_hook(hook, j + 1, st);
-        if (dd) {   // SV[:, j] = sigma_j S w_j, SAV[:, j] = sigma_j S y_j
-            SrdctCols cols{};
-            cols.ncols = 2;
-            cols.x[0] = c.V + (size_t)(c.vring ? j % c.vring : j) * c.ldv;
-            cols.x[1] = c.Y;
-            cols.out[0] = c.SV + (size_t)j * c.sp.s;
-            cols.out[1] = c.SAV + (size_t)j * c.sp.s;
-            cols.colscale = c.stepsc + 4 * (size_t)j;
-            cols.iscal = c.iscal;
-            cols.step = j;
-            srdct_launch(*dd, cols, st);
+        // dense sketches of w_j, and of y~ where it is sketched directly (nothing once
+        // the process stopped before step j: a breakdown at step j still needs S w_j)
+        double *wj = c.V + (size_t)(c.vring ? j % c.vring : j) * c.ldv;
+        if (dd) {   // S w_j, and SAV[:, j] = sigma_j S y_j
+            for (int q = 0; q < (ydir ? 2 : 1); ++q) {
+                SrdctCols cols{};
+                cols.ncols = 1;
+                cols.x[0] = q == 0 ? wj : c.Y;
+                cols.out[0] = q == 0 ? c.Sw + (size_t)j * c.sp.s : c.SAV + (size_t)j * c.sp.s;
+                cols.colscale = q == 0 ? nullptr : c.stepsc + 4 * (size_t)j;
+                cols.iscal = c.iscal;
+                cols.step = q == 0 ? j - 1 : j;
+                srdct_launch(*dd, cols, st);
+            }
         }
-        if (sd) {   // S w_j and S y_j (exponents written by the update kernel)
+        if (sd) {   // S w_j, and S y_j (exponents written by the update kernel)
             SrhtCols cols{};
-            cols.ncols = 2;
-            cols.x[0] = c.V + (size_t)(c.vring ? j % c.vring : j) * c.ldv;
+            cols.ncols = ydir ? 2 : 1;
+            cols.x[0] = wj;
             cols.e[0] = c.ews + j;
             cols.part[0] = c.skSV;
             cols.x[1] = c.Y;
             cols.e[1] = c.eys + j;
             cols.part[1] = c.skSAV;
             cols.iscal = c.iscal;
-            cols.step = j;
+            cols.step = j - 1;
             srht_launch(*sd, cols, st);
         }
     }
@@ -834,6 +913,7 @@ skf_status arnoldi_run(const skf_csr *A, const skf_sketch *S, const double *b, i
     c.sk_scale = c.srht ? 1.0 / sqrt((double)S->s) : c.inv_sqrt_zeta;
     c.m = m;
     c.k = k;
+    c.every = hook ? hook->every : 0;
     c.V = V;
     c.ldv = ldv;
     c.vring = vring;
@@ -854,7 +934,7 @@ skf_status arnoldi_run(const skf_csr *A, const skf_sketch *S, const double *b, i
     char *ws = nullptr;
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t szY = sizeof(double) * A->n;
-    const size_t szP1 = sizeof(double) * (size_t)std::max(std::max(G, Gs), pipe_ctas(A->n)) * kP1;
+    const size_t szP1 = sizeof(double) * (size_t)std::max(std::max(G, Gs), pipe_ctas(A->n, S->s)) * kP1;
     const size_t szP2 = sizeof(double) * (size_t)G * kP2;
     const size_t szFd = sizeof(double) * (size_t)m * kP1;
     const size_t szFw = sizeof(double) * (size_t)(m + 1) * 2;
@@ -865,10 +945,12 @@ skf_status arnoldi_run(const skf_csr *A, const skf_sketch *S, const double *b, i
     const size_t szE = sizeof(int) * (size_t)m;
     const size_t szEps = sizeof(double) * (size_t)m;
     c.rs = row_split_of(A);
+    const size_t szSw = c.identity ? 0 : sizeof(double) * (size_t)(m + 1) * S->s;
+    const size_t szCoef = sizeof(double) * (size_t)m * kMaxK;
     const size_t szSeg = sizeof(double) * (size_t)std::max<int64_t>(c.rs.nseg, 1);
     const size_t szDct = c.direct ? srdct_work_bytes(S) : 0;   // FFT form of the SRDCT: its complex buffers
     const size_t total = al(szY) + al(szP1) + al(szP2) + al(szFd) + al(szFw) + al(szSc) + al(szCnt) + 2 * al(szSk) +
-                         al(szGram) + 2 * al(szE) + al(szEps) + al(szSeg) + al(szDct);
+                         al(szGram) + 2 * al(szE) + al(szEps) + al(szSeg) + al(szDct) + al(szSw) + al(szCoef);
     skf_status stt = dalloc((void **)&ws, total, st);
     if (stt != SKF_OK) return stt;
     size_t off = 0;
@@ -891,10 +973,13 @@ skf_status arnoldi_run(const skf_csr *A, const skf_sketch *S, const double *b, i
     c.ews = (int *)take(szE);
     c.epscol = (double *)take(szEps);
     c.seg_part = (double *)take(szSeg);
+    c.Sw = (double *)take(szSw);
+    c.coef = (double *)take(szCoef);
     if (szDct) dd.work = (double2 *)take(szDct);
     cudaMemsetAsync(c.cnt, 0, szCnt, st);
 
-    const size_t smem = c.sparse ? sizeof(int) * 4 * S->s : 0;   // two limbs for each of S v_j, S A v_j
+    // two limbs of S w_j (twice that with S y~)
+    const size_t smem = c.sparse ? sizeof(int) * 2 * (size_t)(c.pattern8 ? 16 * c.p8_block : S->s) : 0;
     k_arnoldi_init<<<G, kThreads, 0, st>>>(c, b);
     call_col_hook(hook, 0, st);
     const SrhtDev *sdp = c.srht ? &sd : nullptr;

@@ -501,6 +501,7 @@ struct RuleDev {
 struct StepHook {
     void (*fn)(void *ctx, int done, cudaStream_t st) = nullptr;
     void *ctx = nullptr;
+    int every = 0;   // fn acts at done = every, 2 every, ... only (0: no fn)
     void (*col_fn)(void *ctx, int j, cudaStream_t st) = nullptr;
     void *col_ctx = nullptr;
 };
