@@ -147,6 +147,7 @@ struct skf_sketch {
     // e^{-2 pi i t / N} for t < N, and per sampled row k the DCT twist
     // e^{-i pi k / (2N)} times the row's scale (device)
     int64_t fft_len = 0;
+    int fft_p1 = 0;                   // > 0: the passes stop at this span, the sampled outputs are summed from there
     int nrad = 0;
     int rad[64] = {};
     double2 *tw = nullptr;
@@ -639,6 +640,7 @@ struct SrdctDev {
     const double *E;        // [n] signs
     const double *costab;   // [4n] cos(pi j / (2n)) (direct form)
     int64_t fft_len;        // FFT form: n / 2 (even n) or n (odd n); 0: direct form
+    int fft_p1;             // pruned form: span after the passes (skf_srdct.cu), 0: all passes
     int nrad;               // Stockham passes of the FFT
     int rad[64];
     const double2 *tw;      // [n] e^{-2 pi i t / n}
