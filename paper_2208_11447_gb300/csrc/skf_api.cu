@@ -476,8 +476,9 @@ static skf_status run_arnoldi(const skf_csr *A, const skf_sketch *S, const doubl
 // hook at p = d, 2d, ... < m as soon as the leading p columns are final.
 struct StopCtx {
     skf_method method;
-    int s, m, d, next_p;
-    const double *vscale, *SV, *SAV;
+    int s, m, d, next_p, kt;
+    skf_dtype vdt;
+    const double *vscale, *SV, *SAV, *H;
     int *iscal, *iscal_chk;
     double *sf_prev, *sf_cur, *state;
     const RuleDev *rule;
@@ -524,7 +525,8 @@ static void stop_hook(void *ctx, int done, cudaStream_t st) {
     while (k->err == SKF_OK && k->next_p <= done && k->next_p < k->m) {
         const int p = k->next_p;
         k->next_p += k->d;
-        k->err = stop_check(k->method, k->s, p, k->vscale, k->SV, k->SAV, k->iscal, k->iscal_chk, k->sf_prev,
+        k->err = stop_check(k->method, k->s, p, k->vdt, k->vscale, k->SV, k->SAV, k->H, k->m + 1, k->kt, k->iscal,
+                            k->iscal_chk, k->sf_prev,
                             k->sf_cur, k->state, *k->rule, k->tol_quad, k->stop_tol, st);
     }
 }
@@ -614,6 +616,9 @@ static skf_status solve_enqueue(skf_method method, const skf_csr *A, const skf_s
         sc.vscale = vscale;
         sc.SV = SV;
         sc.SAV = SAV;
+        sc.vdt = bt;
+        sc.H = H;
+        sc.kt = p.k;
         sc.iscal = iscal;
         sc.rule = &rule;
         sc.tol_quad = p.tol;

@@ -597,9 +597,11 @@ skf_status accumulate_column(const void *w, skf_dtype vdt, const double *z, cons
 // the tail of the leading p columns in sketched form, then the comparison
 // with the previous checkpoint; on success sets iscal to stop at m_eff = p.
 // Work buffers: iscal_chk[4], sf_prev[s], sf_cur[s], state[4] ([0] previous
-// checkpoint valid, [1] last estimate, [2] stop step), zeroed by the caller.
-skf_status stop_check(skf_method method, int s, int p, const double *vscale, const double *SV, const double *SAV,
-                      int *iscal, int *iscal_chk, double *sf_prev, double *sf_cur, double *state, const RuleDev &rule,
+// checkpoint valid, [1] last estimate, [2] stop step, [3] eps), zeroed by the
+// caller.
+// H, ldh, kt: as for tail_run (the relation form, with a basis of type vdt).
+skf_status stop_check(skf_method method, int s, int p, skf_dtype vdt, const double *vscale, const double *SV,
+                      const double *SAV, const double *H, int ldh, int kt, int *iscal, int *iscal_chk, double *sf_prev, double *sf_cur, double *state, const RuleDev &rule,
                       double tol_quad, double stop_tol, cudaStream_t st);
 
 // SRHT sketch (see skf_srht.cu): blocks of 2^b entries transformed exactly in

@@ -81,11 +81,11 @@ __global__ void k_tail_copy(const double *__restrict__ SV, const double *__restr
         const int64_t r = idx % c.s;
         double v = 0.0;
         if (col < me) v = SV[r + (int64_t)col * c.s];
-        else if (c.rel ? col == me : col < 2 * me) v = SAV[r + (int64_t)(c.rel ? me - 1 : col - me) * c.s];
+        else if (c.rel ? (col == me && me > 0) : col < 2 * me) v = SAV[r + (int64_t)(c.rel ? me - 1 : col - me) * c.s];
         c.Aw[idx] = v;
     }
     if (blockIdx.x == 0 && threadIdx.x < 8) c.qstate[threadIdx.x] = 0.0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *c.lev_cnt = 0u;
+    if (blockIdx.x == 0 && threadIdx.x < 2) c.lev_cnt[threadIdx.x] = 0u;
 }
 
 // Householder reflector for column jj (LAPACK convention: beta = -sign(x0)
@@ -171,52 +171,78 @@ __global__ void __launch_bounds__(kHhThreads) k_householder(TailCtx c, int jj) {
 // that CTA's shared memory until the end, so a CTA's trailing columns are
 // only ever read and updated on chip.  The only data a step needs from
 // another CTA is its pivot column: the owner of column jj + 1 updates that
-// column first at step jj, writes it to global memory and publishes it (a
-// release store of jj + 1 to a step counter); every other CTA starts step
-// jj + 1 as soon as the counter reaches jj + 1 (bounded wait), so the updates
-// of the remaining columns overlap the next steps instead of meeting at a
-// grid barrier.  Each step is one pass over the pivot column per CTA:
+// column first at step jj and publishes it while it writes it; the updates of
+// the remaining columns overlap the next steps instead of meeting at a grid
+// barrier.  Each step is one pass over the pivot column per CTA:
 // ||x(jj+1:)||^2 and the products x(jj+1:)^T y for the CTA's columns, summed
-// in one block reduction; the reflector (LAPACK convention, as
-// k_householder) is formed identically by every CTA.
+// in one block reduction; the reflector (that of k_householder) is formed
+// identically by every CTA.
+//
+// The factorisation is one chain of hand-offs between CTAs, so its time is the
+// latency of one of them.  A published column carries its own flag: the
+// publish buffer starts as all-ones words (a NaN no arithmetic produces), each
+// thread polls the entries it needs itself (relaxed 8-byte loads, bounded
+// wait: SKF_ERR_TIMEOUT), and nothing is fenced.  A column followed by a
+// released counter, polled by one thread before the column is loaded, costs
+// one more round trip to L2 and a fence: 4.2 -> 3.4 us per reflector (s = 800, 201
+// reflectors: 849 -> 680 us; s = 160, 41: 150 -> 115 us).  Of the 3.1 us (stamps)
+// 0.8 pass until the column is there, 0.65 in the two sums, 1.1 in the reflector's
+// scalars (rsqrt and reciprocal; refining single-precision seeds instead was
+// slower, 790 us: the conversions use the FP64 pipe), 0.5 in the update.  Sums
+// formed while loading (788 us), 512 threads and naps between polls were slower.
 constexpr int kQrThreads = 256;
 constexpr int kQrOwn = 7;            // columns per CTA (at most)
 constexpr long long kQrBudget = 1ll << 31;
+constexpr int kQrPoll = 4;           // entries of the pivot column a thread polls at a time
 
-__device__ __forceinline__ unsigned qr_ld_acquire(const unsigned *p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+constexpr unsigned long long kQrEmpty = ~0ull;   // entry not yet published
+
+__device__ __forceinline__ unsigned long long qr_ld(const double *p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void qr_publish(double *p, double x) {
+    unsigned long long v = (unsigned long long)__double_as_longlong(x);
+    if (v == kQrEmpty) v = 0x7FF8000000000000ull;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
 
-// sums over the CTA of nv <= kQrOwn + 1 per-thread values, in a fixed order,
-// into tot[] (visible to every thread on return)
+// sums over the CTA of nv <= kQrOwn + 1 per-thread values, in a fixed order.
+// Every value is added up by 8 / 4 / 2 warps' worth of partial sums (few
+// dependent FP64 additions: 65 cycles each) that qr_total combines.
+__device__ __forceinline__ int qr_parts(int nv) { return nv <= 2 ? 4 : nv <= 4 ? 2 : 1; }
 __device__ __forceinline__ void qr_block_sums(const double (&v)[kQrOwn + 1], int nv, double *sm, double *tot) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll
     for (int k = 0; k < kQrOwn + 1; ++k)
         if (k < nv) sm[k * kQrThreads + tid] = v[k];
     __syncthreads();
-    if (warp < nv) {
-        double a = 0.0;
-#pragma unroll
-        for (int r = 0; r < kQrThreads / 32; ++r) a += sm[warp * kQrThreads + lane + 32 * r];
+    const int np = qr_parts(nv), val = warp / np, len = kQrThreads / np;
+    if (val < nv) {
+        const double *p = sm + val * kQrThreads + (warp % np) * len + lane;
+        double a = p[0];
+        for (int r = 32; r < len; r += 32) a += p[r];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
         if (lane == 0) tot[warp] = a;
     }
     __syncthreads();
 }
-
-size_t qr_smem_bytes(int s) {
-    return sizeof(double) * ((size_t)kQrOwn * s + s + (size_t)(kQrOwn + 1) * kQrThreads + kQrOwn + 1);
+__device__ __forceinline__ double qr_total(const double *tot, int nv, int k) {
+    const int np = qr_parts(nv);
+    const double *p = tot + k * np;
+    return np == 4 ? (p[0] + p[1]) + (p[2] + p[3]) : np == 2 ? p[0] + p[1] : p[0];
 }
 
-__global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, unsigned *ready, int *flag) {
+size_t qr_smem_bytes(int s) {
+    return sizeof(double) * ((size_t)kQrOwn * s + s + (size_t)(kQrOwn + 1) * kQrThreads + kQrThreads / 32);
+}
+
+__global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, double *pub, int *flag) {
     extern __shared__ double qsm[];
-    __shared__ int ok;
-    __shared__ double qsc[2];                     // tau, scale of the current reflector
-    __shared__ double qf[kQrOwn], qfs[kQrOwn];    // f and f scale of the columns being updated
+    __shared__ double qsc[2];       // u_0 and 1 / D of the current reflector
+    __shared__ double qf[kQrOwn];   // factors f of the columns being updated
     const int me = c.iscal[1];
     const int ncols = c.rel ? me + 1 : 2 * me;
     const int s = c.s;
@@ -233,45 +259,61 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, unsigned *
     for (int k = 0; k < nq; ++k)
         for (int i = tid; i < s; i += kQrThreads) cols[(size_t)k * s + i] = c.Aw[i + (int64_t)(g + k * G) * s];
     __syncthreads();
+    int kf = 0, cf = g;   // own columns that trail the pivot: k >= kf; column kf is cf = g + kf G
     for (int jj = 0; jj < nref; ++jj) {
-        // own columns that trail the pivot: k >= kf (column g + k G > jj)
-        const int kf = jj < g ? 0 : (jj - g) / G + 1;
-        const bool writer = (jj % G) == g;                 // owns the pivot column
-        if (kf >= nq && !writer) continue;
-        // pivot column jj, rows jj .. s-1
+        const bool writer = jj == cf && kf < nq;           // owns the pivot column
         if (writer) {
-            const double *xc = cols + (size_t)((jj - g) / G) * s;
-            for (int i = jj + tid; i < s; i += kQrThreads) xs[i] = xc[i];
-        } else {
-            if (tid == 0) {
-                const long long t0 = clock64();
-                int good = 1;
-                while (qr_ld_acquire(ready) < (unsigned)jj) {
-                    if (*(volatile int *)flag != 0 || clock64() - t0 > kQrBudget) {
-                        good = 0;
-                        break;
-                    }
-                }
-                if (!good) atomicExch(flag, 1);
-                ok = good;
-            }
-            __syncthreads();
-            if (!ok) {
-                if (tid == 0) atomicExch(&c.iscal[2], (int)SKF_ERR_TIMEOUT);
-                return;
-            }
-            const double *x = c.Aw + (int64_t)jj * s;
-            for (int i = jj + tid; i < s; i += kQrThreads) xs[i] = __ldcg(x + i);
+            ++kf;
+            cf += G;
         }
-        __syncthreads();
-        const double x0 = xs[jj];
+        if (kf >= nq && !writer) continue;
         // the next pivot column (jj + 1) is this CTA's first trailing one:
         // update and publish it before the others
-        const bool pivot_owner = kf < nq && g + kf * G == jj + 1;
+        const bool pivot_owner = kf < nq && cf == jj + 1;
         const int n1 = pivot_owner ? 1 : nq - kf;
         double loc[kQrOwn + 1];
 #pragma unroll
         for (int k = 0; k < kQrOwn + 1; ++k) loc[k] = 0.0;
+        // pivot column jj, rows jj .. s-1, into xs
+        bool late = false;
+        if (writer) {
+            const double *xc = cols + (size_t)(kf - 1) * s;
+            for (int i = jj + tid; i < s; i += kQrThreads) xs[i] = xc[i];
+        } else if (jj == 0) {
+            for (int i = tid; i < s; i += kQrThreads) xs[i] = c.Aw[i];   // column 0 is not modified
+        } else {
+            const double *x = pub + (int64_t)jj * s;
+            const long long t0 = clock64();
+            // a thread's entries are polled together (one after another, each a round
+            // trip to L2, took 0.6 us more per reflector at s = 800)
+            for (int i0 = jj + tid; i0 < s; i0 += kQrPoll * kQrThreads) {
+                unsigned long long v[kQrPoll];
+                bool empty = true;
+                for (int n = 1; empty && !late; ++n) {
+                    empty = false;
+#pragma unroll
+                    for (int u = 0; u < kQrPoll; ++u) {
+                        const int i = i0 + u * kQrThreads;
+                        v[u] = i < s ? qr_ld(x + i) : 0ull;
+                    }
+#pragma unroll
+                    for (int u = 0; u < kQrPoll; ++u) empty = empty || v[u] == kQrEmpty;
+                    if ((n & 63) == 0) late = clock64() - t0 > kQrBudget || *(volatile int *)flag != 0;
+                }
+#pragma unroll
+                for (int u = 0; u < kQrPoll; ++u) {
+                    const int i = i0 + u * kQrThreads;
+                    if (i < s) xs[i] = __longlong_as_double((long long)v[u]);
+                }
+            }
+        }
+        if (__syncthreads_or(late)) {
+            if (tid == 0) {
+                atomicExch(flag, 1);
+                atomicExch(&c.iscal[2], (int)SKF_ERR_TIMEOUT);
+            }
+            return;
+        }
         for (int i = jj + 1 + tid; i < s; i += kQrThreads) {
             const double xi = xs[i];
             loc[0] = fma(xi, xi, loc[0]);
@@ -279,64 +321,64 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, unsigned *
             for (int k = 0; k < kQrOwn; ++k)
                 if (k < n1) loc[1 + k] = fma(xi, cols[(size_t)(kf + k) * s + i], loc[1 + k]);
         }
-        qr_block_sums(loc, 1 + (kf < nq ? n1 : 0), sm, tot);
-        // The reflector (from one rsqrt and one reciprocal: with
-        // r = (x0^2 + sig)^-1/2, ||x|| = (x0^2 + sig) r, beta = -sign(x0) ||x||,
-        // tau = (beta - x0) / beta = 1 + |x0| r, 1 / (x0 - beta) =
-        // sign(x0) / (|x0| + ||x||)) and the factors f = tau (y(jj) + scale x^T y)
-        // of the columns, by warp 0 only: a warp instruction occupies the FP64
-        // pipe for 16 cycles whatever its active lanes, so scalar FP64 work
+        const int nv1 = 1 + (kf < nq ? n1 : 0);
+        qr_block_sums(loc, nv1, sm, tot);
+        const double x0 = xs[jj];
+        // The reflector, unnormalised, from one rsqrt and one reciprocal: with
+        // r = (x0^2 + sig)^-1/2, ||x|| = (x0^2 + sig) r and u = [x0 + sign(x0) ||x||;
+        // x(jj+1:)], H = I - u u^T / D, D = ||x|| (||x|| + |x0|), and the factor of
+        // a column y is f = (u_0 y(jj) + x^T y) / D (a quotient with the LAPACK
+        // scaling of u and its two more products were half of the 1.3 us this
+        // takes on the chain).  By warp 0 only: a warp instruction occupies the
+        // FP64 pipe for 16 cycles whatever its active lanes, so scalar FP64 work
         // repeated by every warp costs eight times the pipe time.
         if (warp0) {
-            const double sig = tot[0];
-            double tau = 0.0, beta = x0, scale = 0.0;
+            const double sig = qr_total(tot, nv1, 0);
+            const bool upd = lane < n1 && kf < nq;
+            const double xy = upd ? qr_total(tot, nv1, 1 + lane) : 0.0;
+            const double yj = upd ? cols[(size_t)(kf + lane) * s + jj] : 0.0;
+            double beta = x0, u0 = 0.0, di = 0.0;
             if (sig > 0.0 || x0 == 0.0) {
                 const double q2 = fma(x0, x0, sig);
                 if (q2 > 0.0) {
                     const double r = rsqrt(q2);
-                    const double nx = q2 * r;
-                    const double sgn = x0 >= 0.0 ? 1.0 : -1.0;
-                    beta = -sgn * nx;
-                    tau = fma(fabs(x0), r, 1.0);
-                    scale = sgn / (fabs(x0) + nx);
+                    const double nx = x0 >= 0.0 ? q2 * r : -(q2 * r);
+                    di = 1.0 / fma(x0, nx, q2);
+                    u0 = x0 + nx;
+                    beta = -nx;
                 }
             }
             if (lane == 0) {
-                qsc[0] = tau;
-                qsc[1] = scale;
+                qsc[0] = u0;
+                qsc[1] = di;
                 if (writer) c.Rdiag[jj] = beta;
             }
-            if (lane < n1 && kf < nq) {
-                const double f = tau * (cols[(size_t)(kf + lane) * s + jj] + scale * tot[1 + lane]);
-                qf[lane] = f;
-                qfs[lane] = f * scale;
-            }
+            if (upd) qf[lane] = fma(u0, yj, xy) * di;
         }
         __syncthreads();
         if (kf >= nq) continue;
-        const double tau = qsc[0];
-        // y(jj) -= f, y(i) -= f scale x_i
-        if (tau != 0.0) {
-#pragma unroll
-            for (int k = 0; k < kQrOwn; ++k) {
-                if (k < n1) {
-                    double *y = cols + (size_t)(kf + k) * s;
-                    const double fs = qfs[k];
-                    for (int i = jj + 1 + tid; i < s; i += kQrThreads) y[i] = fma(-fs, xs[i], y[i]);
-                    if (tid == 0) y[jj] -= qf[k];
-                }
-            }
-        }
+        const double u0 = qsc[0], di = qsc[1];   // di = 0: no reflection
+        // y(jj) -= f u_0, y(i) -= f x_i; the next pivot column is published as it
+        // is written (rows jj + 1 .. s - 1: what the next reflector reads)
         if (pivot_owner) {
-            // publish column jj + 1 (rows jj + 1 .. s - 1: what the next reflector reads)
-            __syncthreads();
-            double *yg = c.Aw + (int64_t)(jj + 1) * s;
-            const double *y = cols + (size_t)kf * s;
-            for (int i = jj + 1 + tid; i < s; i += kQrThreads) yg[i] = y[i];
-            __syncthreads();
-            if (tid == 0) {
-                __threadfence();
-                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ready), "r"((unsigned)(jj + 1)) : "memory");
+            double *y = cols + (size_t)kf * s, *yp = pub + (int64_t)(jj + 1) * s;
+            const double f = qf[0];
+            for (int i0 = jj + tid; i0 < s; i0 += kQrPoll * kQrThreads) {
+                double v[kQrPoll];
+#pragma unroll
+                for (int u = 0; u < kQrPoll; ++u) {
+                    const int i = i0 + u * kQrThreads;
+                    v[u] = i < s ? y[i] : 0.0;
+                    if (i < s && di != 0.0) v[u] = fma(-f, i > jj ? xs[i] : u0, v[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < kQrPoll; ++u) {
+                    const int i = i0 + u * kQrThreads;
+                    if (i < s) {
+                        if (i > jj) qr_publish(yp + i, v[u]);
+                        y[i] = v[u];
+                    }
+                }
             }
             const int n2 = nq - kf - 1;
             if (n2 > 0) {   // the rest of this CTA's trailing columns
@@ -348,23 +390,31 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, unsigned *
                     for (int k = 0; k < kQrOwn; ++k)
                         if (k < n2) loc[k] = fma(xi, cols[(size_t)(kf + 1 + k) * s + i], loc[k]);
                 }
+                __syncthreads();   // (qf[0] has been read by every thread)
                 qr_block_sums(loc, n2, sm, tot);
-                if (warp0 && lane < n2) {
-                    const double f = tau * (cols[(size_t)(kf + 1 + lane) * s + jj] + qsc[1] * tot[lane]);
-                    qf[lane] = f;
-                    qfs[lane] = f * qsc[1];
-                }
+                if (warp0 && lane < n2)
+                    qf[lane] = fma(u0, cols[(size_t)(kf + 1 + lane) * s + jj], qr_total(tot, n2, lane)) * di;
                 __syncthreads();
-                if (tau != 0.0) {
+                if (di != 0.0) {
 #pragma unroll
                     for (int k = 0; k < kQrOwn; ++k) {
                         if (k < n2) {
-                            double *y = cols + (size_t)(kf + 1 + k) * s;
-                            const double fs = qfs[k];
-                            for (int i = jj + 1 + tid; i < s; i += kQrThreads) y[i] = fma(-fs, xs[i], y[i]);
-                            if (tid == 0) y[jj] -= qf[k];
+                            double *yk = cols + (size_t)(kf + 1 + k) * s;
+                            const double fk = qf[k];
+                            for (int i = jj + 1 + tid; i < s; i += kQrThreads) yk[i] = fma(-fk, xs[i], yk[i]);
+                            if (tid == 0) yk[jj] = fma(-fk, u0, yk[jj]);
                         }
                     }
+                }
+            }
+        } else if (di != 0.0) {
+#pragma unroll
+            for (int k = 0; k < kQrOwn; ++k) {
+                if (k < n1) {
+                    double *y = cols + (size_t)(kf + k) * s;
+                    const double f = qf[k];
+                    for (int i = jj + 1 + tid; i < s; i += kQrThreads) y[i] = fma(-f, xs[i], y[i]);
+                    if (tid == 0) y[jj] = fma(-f, u0, y[jj]);
                 }
             }
         }
@@ -509,7 +559,7 @@ __device__ __forceinline__ double warp_sumsq(const double (&x)[K]) {
 // R_11 in compact form: RT (row-major), RTs = D^{-1} R (row-major) and
 // Rcs = R D^{-1} (column-major), ld m, upper triangles with the diagonal;
 // rinv = 1 / R_jj (0 for a zero pivot, which sets qstate[7]); cn2[q] =
-// ||R(:, q)||^2 (thread q, in row order).
+// ||R(:, q)||^2; in the relation form gamma = R(m+1, m+1) / R(m, m) (qstate[6]).
 __global__ void __launch_bounds__(kThreads) k_r_pack(TailCtx c) {
     const int me = c.iscal[1];
     const int m = c.m;
@@ -528,14 +578,91 @@ __global__ void __launch_bounds__(kThreads) k_r_pack(TailCtx c) {
         c.RTs[q + (int64_t)i * m] = vr;
         c.Rcs[i + (int64_t)q * m] = vc;
     }
-    if (gid < me) {
-        const int q = (int)gid;
-        const double d = c.Rdiag[q];
-        c.rinv[q] = d != 0.0 ? 1.0 / d : 0.0;
-        if (!(d != 0.0)) c.qstate[7] = 1.0;
+    // 1 / R_jj, squared column norms (one warp per column; a thread per column,
+    // 240 dependent loads and FMAs long, took 24 us at m = 240: 7.5 us)
+    const int lane = threadIdx.x & 31;
+    for (int64_t q = gid >> 5; q < me; q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         double a2 = 0.0;
-        for (int i = 0; i < q; ++i) a2 = fma(c.Aw[i + (int64_t)q * c.s], c.Aw[i + (int64_t)q * c.s], a2);
-        c.cn2[q] = fma(d, d, a2);
+        for (int i = lane; i < q; i += 32) a2 = fma(c.Aw[i + q * c.s], c.Aw[i + q * c.s], a2);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+        if (lane == 0) {
+            const double d = c.Rdiag[q];
+            c.rinv[q] = d != 0.0 ? 1.0 / d : 0.0;
+            if (!(d != 0.0)) c.qstate[7] = 1.0;
+            c.cn2[q] = fma(d, d, a2);
+            if (q == me - 1)   // gamma of the relation form
+                c.qstate[6] = (c.rel && c.method == SKF_METHOD_SGMRES && d != 0.0) ? c.Rdiag[me] / d : 0.0;
+        }
+    }
+}
+
+// The estimate of cond(R) (qstate[5]) and the diagonal ratio (qstate[3]) by
+// the first two warps of a CTA (every thread calls): ||R^{-1}|| LINPACK-style
+// (warp 0) times the largest column norm of R (warp 1, with the extreme
+// diagonal entries).
+template <int K>
+__device__ void cond_estimate(const TailCtx &c, double *qs2) {
+    __shared__ double res[4];
+    const int me = c.iscal[1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int m = c.m;
+    const int ka = (me + 31) >> 5;
+    if (warp == 0) {
+        double z[K];
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk) z[kk] = 0.0;
+        double r = INFINITY;
+        if (c.qstate[7] == 0.0 && me > 0) {
+            warp_row_solve<K, true>(c.RTs, me, m, z);   // z' = D z, R^T z = b
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) {
+                const int i = lane + 32 * kk;
+                z[kk] = (kk < ka && i < me) ? z[kk] * c.rinv[i] : 0.0;
+            }
+            const double zn = warp_sumsq(z);
+            warp_back_solve<K>(c.Rcs, me, m, z);         // y' = D y, R y = z
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) {
+                const int i = lane + 32 * kk;
+                z[kk] = (kk < ka && i < me) ? z[kk] * c.rinv[i] : 0.0;
+            }
+            const double yn = warp_sumsq(z);
+            r = zn > 0.0 ? sqrt(yn / zn) : 0.0;
+        }
+        if (lane == 0) res[0] = r;
+    } else if (warp == 1) {
+        double mx = 0.0, mn = INFINITY, mxd = 0.0;
+        for (int q = lane; q < me; q += 32) {
+            const double d = fabs(c.Rdiag[q]);
+            mx = fmax(mx, c.cn2[q]);
+            mn = fmin(mn, d);
+            mxd = fmax(mxd, d);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            mxd = fmax(mxd, __shfl_xor_sync(0xffffffffu, mxd, o));
+        }
+        if (lane == 0) {
+            res[1] = sqrt(mx);
+            res[2] = mn;
+            res[3] = mxd;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double mn = res[2], mxd = res[3];
+        // never less than the diagonal ratio, a lower bound of cond(R)
+        const double ratio = mxd > 0.0 ? mn / mxd : 0.0;
+        const double cond = me == 0 ? 0.0 : fmax(res[0] * res[1], mn > 0.0 ? mxd / mn : INFINITY);
+        c.qstate[3] = ratio;
+        c.qstate[5] = cond;
+        if (qs2) {   // a second method on the same whitening
+            qs2[3] = ratio;
+            qs2[5] = cond;
+        }
     }
 }
 
@@ -543,9 +670,8 @@ __global__ void __launch_bounds__(kThreads) k_r_pack(TailCtx c) {
 // (relation form: T = [R_11 H(1:m, 1:m-1), R(1:m, m+1)] -> M only).  Two
 // warps per CTA, so that the rows spread over the SMs (each step is a few
 // FP64 instructions per warp; more warps per SM would queue on the FP64
-// pipe).  The last CTA computes meanwhile the estimate of cond(R) (qstate[5]):
-// ||R^{-1}|| LINPACK-style (warp 0) times the largest column norm of R (warp
-// 1), and, in the relation form, gamma = R(m+1, m+1) / R(m, m) (qstate[6]).
+// pipe).  Where the node solves are not the Givens ones (which take it along),
+// one more CTA estimates cond(R) meanwhile.
 template <int K>
 __global__ void __launch_bounds__(64) k_tri_right(TailCtx c, int nblk_rows) {
     const int me = c.iscal[1];
@@ -553,51 +679,8 @@ __global__ void __launch_bounds__(64) k_tri_right(TailCtx c, int nblk_rows) {
     const int m = c.m;
     const int ka = (me + 31) >> 5;
     const bool gm = c.method == SKF_METHOD_SGMRES;
-    if ((int)blockIdx.x == nblk_rows) {   // the cond(R) estimate
-        __shared__ double res[2];
-        const bool zp = c.qstate[7] != 0.0;
-        if (warp == 0) {
-            double z[K];
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) z[kk] = 0.0;
-            double r = INFINITY;
-            if (!zp && me > 0) {
-                warp_row_solve<K, true>(c.RTs, me, m, z);   // z' = D z, R^T z = b
-#pragma unroll
-                for (int kk = 0; kk < K; ++kk) {
-                    const int i = lane + 32 * kk;
-                    z[kk] = (kk < ka && i < me) ? z[kk] * c.rinv[i] : 0.0;
-                }
-                const double zn = warp_sumsq(z);
-                warp_back_solve<K>(c.Rcs, me, m, z);         // y' = D y, R y = z
-#pragma unroll
-                for (int kk = 0; kk < K; ++kk) {
-                    const int i = lane + 32 * kk;
-                    z[kk] = (kk < ka && i < me) ? z[kk] * c.rinv[i] : 0.0;
-                }
-                const double yn = warp_sumsq(z);
-                r = zn > 0.0 ? sqrt(yn / zn) : 0.0;
-            }
-            if (lane == 0) res[0] = r;
-        } else {
-            double mx = 0.0;
-            for (int q = lane; q < me; q += 32) mx = fmax(mx, c.cn2[q]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            if (lane == 0) res[1] = sqrt(mx);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double mn = INFINITY, mxd = 0.0;
-            for (int a2 = 0; a2 < me; ++a2) {
-                mn = fmin(mn, fabs(c.Rdiag[a2]));
-                mxd = fmax(mxd, fabs(c.Rdiag[a2]));
-            }
-            c.qstate[3] = mxd > 0.0 ? mn / mxd : 0.0;
-            // never less than the diagonal ratio, a lower bound of cond(R)
-            c.qstate[5] = me == 0 ? 0.0 : fmax(res[0] * res[1], mn > 0.0 ? mxd / mn : INFINITY);
-            c.qstate[6] = (c.rel && gm && me > 0 && c.Rdiag[me - 1] != 0.0) ? c.Rdiag[me] / c.Rdiag[me - 1] : 0.0;
-        }
+    if ((int)blockIdx.x == nblk_rows) {
+        cond_estimate<K>(c, nullptr);
         return;
     }
     const int row = blockIdx.x * 2 + warp;
@@ -638,11 +721,28 @@ __global__ void __launch_bounds__(64) k_tri_right(TailCtx c, int nblk_rows) {
     }
 }
 
+// A second method's tail on the shared whitening: its state starts from the
+// first method's (rdiag ratio, cond(R) estimate, gamma, zero-pivot flag;
+// convergence fields cleared), and a failure of the shared part (a QR
+// timeout) is carried over to its status.
+__device__ __forceinline__ void fork_state(const double *q0, double *q1, const int *isc0, int *isc1) {
+    if (threadIdx.x < 8) {
+        const int i = threadIdx.x;
+        q1[i] = (i == 3 || i >= 5) ? q0[i] : 0.0;
+    }
+    if (threadIdx.x == 0 && isc1[2] == SKF_OK && isc0[2] == SKF_ERR_TIMEOUT) isc1[2] = SKF_ERR_TIMEOUT;
+}
+
+__global__ void k_fork_state(const double *q0, double *q1, const int *isc0, int *isc1) {
+    fork_state(q0, q1, isc0, isc1);
+}
+
 // B = M + M^T, C = M^T M (+ R2^T R2; relation form: + gamma^2 e_m e_m^T)
 // for the Cholesky node solves (not needed by the Givens ones), the
 // transposes, c = ||b|| R_11 e_1, M^T c.
-__global__ void __launch_bounds__(kThreads) k_tail_prep(TailCtx c) {
+__global__ void __launch_bounds__(kThreads) k_tail_prep(TailCtx c, double *qs2, int *iscal2) {
     const int me = c.iscal[1];
+    if (qs2 && blockIdx.x == 0) fork_state(c.qstate, qs2, c.iscal, iscal2);
     const int64_t tot = (int64_t)me * me;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; !c.hess && idx < tot;
          idx += (int64_t)gridDim.x * blockDim.x) {
@@ -1204,9 +1304,20 @@ __global__ void __launch_bounds__(kNodeThreads) k_nodes_g(TailCtx c, int n0, int
 // groups are unrolled, so the pivot's register is known at compile time.
 constexpr int kHessWarps = 4;   // nodes (warps) per CTA
 
+// The contexts of the one or two methods of a tail (blockIdx.y).
+struct TailMethods {
+    TailCtx c[2];
+};
+
 template <int K>
-__global__ void __launch_bounds__(32 * kHessWarps) k_nodes_hess(TailCtx c, int n0, int off, int nn, double *Rs,
-                                                                 size_t rstride) {
+__global__ void __launch_bounds__(32 * kHessWarps) k_nodes_hess(TailMethods tm, int n0, int off, int nn,
+                                                                 size_t rstride, int est) {
+    const TailCtx &c = tm.c[blockIdx.y];
+    if (est && blockIdx.x == gridDim.x - 1) {   // first launch: cond(R), beside the node solves
+        if (blockIdx.y == 0) cond_estimate<K>(c, gridDim.y > 1 ? tm.c[1].qstate : nullptr);
+        return;
+    }
+    double *Rs = c.Nw;
     const int me = c.iscal[1];
     if (c.qstate[0] != 0.0 || me == 0) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1432,9 +1543,9 @@ __global__ void __launch_bounds__(kNodeThreads) k_nodes_cplx(TailCtx c, int n0, 
 // Sum the node solutions of each level of the batch (CTA i: level lev0 + i,
 // four interleaved partial sums over its nodes, added in a fixed order), then
 // the last CTA to finish runs the acceptance test of Sec. 4.1 level by level.
-__global__ void __launch_bounds__(kThreads) k_levels(TailCtx c, int lev0, int nlev, const int *lev_start,
+__global__ void __launch_bounds__(kThreads) k_levels(TailMethods tm, int lev0, int nlev, const int *lev_start,
                                                      const int *lev_ell, int n0, double tol, int last_batch) {
-    __shared__ double red[64];
+    const TailCtx &c = tm.c[blockIdx.y];
     __shared__ int is_last;
     const int me = c.iscal[1];
     if (c.qstate[0] != 0.0 || me == 0) return;
@@ -1446,6 +1557,18 @@ __global__ void __launch_bounds__(kThreads) k_levels(TailCtx c, int lev0, int nl
         for (int a = threadIdx.x; a < me; a += blockDim.x) {
             double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
             int nd = a0;
+            for (; nd + 15 < a1; nd += 16) {   // 16 loads in flight (4 at a time 55 us, now 43, over the five launches at m = 40)
+                double o[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) o[u] = c.out[(size_t)(nd + u) * m + a];
+#pragma unroll
+                for (int u = 0; u < 16; u += 4) {
+                    p0 += o[u];
+                    p1 += o[u + 1];
+                    p2 += o[u + 2];
+                    p3 += o[u + 3];
+                }
+            }
             for (; nd + 3 < a1; nd += 4) {
                 p0 += c.out[(size_t)nd * m + a];
                 p1 += c.out[(size_t)(nd + 1) * m + a];
@@ -1463,39 +1586,53 @@ __global__ void __launch_bounds__(kThreads) k_levels(TailCtx c, int lev0, int nl
     if (!is_last) return;
     __threadfence();
     if (threadIdx.x == 0) *c.lev_cnt = 0u;   // ready for the next batch
-    for (int l = lev0; l < lev0 + nlev; ++l) {
-        const double *ql = c.qbuf + (size_t)l * m;
-        bool accept = false;
-        double rel = 0.0;
-        if (c.nlevels == 1) {
-            accept = true;
-        } else if (l > 0) {
-            const double *qp = c.qbuf + (size_t)(l - 1) * m;
-            double v[2] = {0.0, 0.0};
-            for (int a = threadIdx.x; a < me; a += blockDim.x) {
+    // ||q_l - q_{l-1}||^2 and ||q_l||^2, one warp per level; then the test of
+    // Sec. 4.1 in schedule order (a block sum per level in turn took 10 us
+    // more, over the five launches of a tail)
+    __shared__ double nd2[kThreads / 32], nq2[kThreads / 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int lb = lev0; lb < lev0 + nlev; lb += kThreads / 32) {
+        const int l = lb + warp;
+        if (l < lev0 + nlev) {
+            const double *ql = c.qbuf + (size_t)l * m, *qp = c.qbuf + (size_t)(l > 0 ? l - 1 : 0) * m;
+            double d2 = 0.0, q2 = 0.0;
+            for (int a = lane; a < me; a += 32) {
                 const double qa = __ldcg(ql + a);
                 const double d = qa - __ldcg(qp + a);
-                v[0] = fma(d, d, v[0]);
-                v[1] = fma(qa, qa, v[1]);
+                d2 = fma(d, d, d2);
+                q2 = fma(qa, qa, q2);
             }
-            block_sum<2>(v, red);
-            __shared__ double sv2[2];
-            if (threadIdx.x == 0) { sv2[0] = v[0]; sv2[1] = v[1]; }
-            __syncthreads();
-            rel = sv2[1] > 0.0 ? sqrt(sv2[0] / sv2[1]) : 0.0;
-            accept = sqrt(sv2[0]) <= tol * sqrt(sv2[1]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+                q2 += __shfl_xor_sync(0xffffffffu, q2, o);
+            }
+            if (lane == 0) {
+                nd2[warp] = d2;
+                nq2[warp] = q2;
+            }
         }
-        const bool final_level = last_batch && (l == lev0 + nlev - 1);
-        if (accept || final_level) {
-            for (int a = threadIdx.x; a < me; a += blockDim.x) c.qacc[a] = __ldcg(ql + a);
-            if (threadIdx.x == 0) {
-                c.qstate[0] = 1.0;
-                c.qstate[1] = (double)lev_ell[l];
-                c.qstate[2] = rel;
-                if (!accept && c.iscal[2] == SKF_OK) c.iscal[2] = SKF_ERR_QUAD_NOT_CONVERGED;
+        __syncthreads();
+        for (int w = 0; w < kThreads / 32 && lb + w < lev0 + nlev; ++w) {
+            const int la = lb + w;
+            bool accept = c.nlevels == 1;
+            double rel = 0.0;
+            if (c.nlevels > 1 && la > 0) {
+                rel = nq2[w] > 0.0 ? sqrt(nd2[w] / nq2[w]) : 0.0;
+                accept = sqrt(nd2[w]) <= tol * sqrt(nq2[w]);
             }
-            __syncthreads();
-            return;
+            const bool final_level = last_batch && (la == lev0 + nlev - 1);
+            if (accept || final_level) {
+                const double *ql = c.qbuf + (size_t)la * m;
+                for (int a = threadIdx.x; a < me; a += blockDim.x) c.qacc[a] = __ldcg(ql + a);
+                if (threadIdx.x == 0) {
+                    c.qstate[0] = 1.0;
+                    c.qstate[1] = (double)lev_ell[la];
+                    c.qstate[2] = rel;
+                    if (!accept && c.iscal[2] == SKF_OK) c.iscal[2] = SKF_ERR_QUAD_NOT_CONVERGED;
+                }
+                return;
+            }
         }
         __syncthreads();
     }
@@ -1505,7 +1642,8 @@ __global__ void __launch_bounds__(kThreads) k_levels(TailCtx c, int lev0, int nl
 // ILL_CONDITIONED when R has a zero pivot or the estimate of cond(R)
 // (k_tri_right) exceeds cond_max.
 template <int K>
-__global__ void __launch_bounds__(32) k_coeffs(TailCtx c) {
+__global__ void __launch_bounds__(32) k_coeffs(TailMethods tm) {
+    const TailCtx &c = tm.c[blockIdx.x];
     const int me = c.iscal[1];
     const int lane = threadIdx.x & 31;
     const bool zero_pivot = c.qstate[7] != 0.0;
@@ -1527,10 +1665,25 @@ __global__ void __launch_bounds__(32) k_coeffs(TailCtx c) {
 __global__ void __launch_bounds__(kThreads) k_recombine(const double *__restrict__ V, int64_t ldv, int64_t n,
                                                         const double *__restrict__ z, const int *iscal,
                                                         double *__restrict__ x) {
+    extern __shared__ double zz[];   // [me]
     const int me = iscal[1];
+    for (int j = threadIdx.x; j < me; j += blockDim.x) zz[j] = z[j];
+    __syncthreads();
+    // kAhead entries of a row in flight per thread: few rows leave few warps, and
+    // then the loads' latency decides (N = 25600, m = 240: 110 -> 38 us)
+    constexpr int kAhead = 16;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
         double acc = 0.0;
-        for (int j = 0; j < me; ++j) acc = fma(V[r + (int64_t)j * ldv], z[j], acc);
+        const double *v = V + r;
+        int j = 0;
+        for (; j + kAhead <= me; j += kAhead) {
+            double w[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) w[u] = v[(int64_t)(j + u) * ldv];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) acc = fma(w[u], zz[j + u], acc);
+        }
+        for (; j < me; ++j) acc = fma(v[(int64_t)j * ldv], zz[j], acc);
         x[r] = acc;
     }
 }
@@ -1551,27 +1704,27 @@ __global__ void __launch_bounds__(kThreads) k_recombine2(const double *__restric
     __syncthreads();
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
         double a0 = 0.0, a1 = 0.0;
-        for (int j = 0; j < me; ++j) {
-            const double v = V[r + (int64_t)j * ldv];
-            a0 = fma(v, zz[2 * j], a0);
-            a1 = fma(v, zz[2 * j + 1], a1);
+        const double *v = V + r;
+        constexpr int kAhead = 8;   // as in k_recombine
+        int j = 0;
+        for (; j + kAhead <= me; j += kAhead) {
+            double w[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) w[u] = v[(int64_t)(j + u) * ldv];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                a0 = fma(w[u], zz[2 * (j + u)], a0);
+                a1 = fma(w[u], zz[2 * (j + u) + 1], a1);
+            }
+        }
+        for (; j < me; ++j) {
+            const double w = v[(int64_t)j * ldv];
+            a0 = fma(w, zz[2 * j], a0);
+            a1 = fma(w, zz[2 * j + 1], a1);
         }
         x0[r] = a0;
         x1[r] = a1;
     }
-}
-
-// A second method's tail on the shared whitening: its state starts from the
-// first method's (rdiag ratio, cond(R) estimate, gamma, zero-pivot flag;
-// convergence fields cleared), and a failure of the shared part (a QR
-// timeout) is carried over to its status.
-__global__ void k_fork_state(const double *__restrict__ q0, double *__restrict__ q1, const int *__restrict__ isc0,
-                             int *__restrict__ isc1) {
-    if (threadIdx.x < 8) {
-        const int i = threadIdx.x;
-        q1[i] = (i == 3 || i >= 5) ? q0[i] : 0.0;
-    }
-    if (threadIdx.x == 0 && isc1[2] == SKF_OK && isc0[2] == SKF_ERR_TIMEOUT) isc1[2] = SKF_ERR_TIMEOUT;
 }
 
 // f = V_m z for an FP32 or BF16 basis.  Each product v z_j is formed exactly
@@ -1614,12 +1767,27 @@ __global__ void __launch_bounds__(kThreads) k_recombine_lp(const TB *__restrict_
 }
 
 // S f = S V y = sum_j S v_j y_j with y_j = z_j / vscale_j (sketched form of
-// the approximant, for the stopping criterion); one thread per row of S.
+// the approximant, for the stopping criterion); one thread per row of S.  The
+// quotients once per CTA and 16 entries of a row in flight (a division per
+// entry and thread: 45 us at p = 100).
 __global__ void __launch_bounds__(kThreads) k_sketch_f(TailCtx c, const double *__restrict__ SV, double *__restrict__ sf) {
+    extern __shared__ double zz[];   // [me]
     const int me = c.iscal[1];
+    for (int j = threadIdx.x; j < me; j += blockDim.x) zz[j] = c.z[j] / c.vscale[j];
+    __syncthreads();
+    constexpr int kAhead = 16;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c.s; i += gridDim.x * blockDim.x) {
         double acc = 0.0;
-        for (int j = 0; j < me; ++j) acc = fma(SV[i + (size_t)j * c.s], c.z[j] / c.vscale[j], acc);
+        const double *v = SV + i;
+        int j = 0;
+        for (; j + kAhead <= me; j += kAhead) {
+            double w[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) w[u] = v[(size_t)(j + u) * c.s];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) acc = fma(w[u], zz[j + u], acc);
+        }
+        for (; j < me; ++j) acc = fma(v[(size_t)j * c.s], zz[j], acc);
         sf[i] = acc;
     }
 }
@@ -1655,26 +1823,34 @@ __global__ void k_check_begin(const int *__restrict__ iscal, int *__restrict__ i
     iscal_chk[3] = p;
 }
 
+// eps = max_{j<p} | ||S v_j||^2 - 1 | (Sec. 4.3) into state[3], one warp per
+// column.  Non-negative doubles order like their bits, and the columns of a
+// checkpoint contain those of the one before, so a running integer maximum
+// gives it in any order.
+__global__ void __launch_bounds__(kThreads) k_check_eps(const double *__restrict__ SV, int s, int p,
+                                                        const int *__restrict__ iscal_chk, double *state) {
+    if (iscal_chk[1] == 0) return;
+    const int lane = threadIdx.x & 31;
+    const int j = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+    if (j >= p) return;
+    double a = 0.0;
+#pragma unroll 8
+    for (int i = lane; i < s; i += 32) a = fma(SV[i + (size_t)j * s], SV[i + (size_t)j * s], a);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0)
+        atomicMax((unsigned long long *)(state + 3), (unsigned long long)__double_as_longlong(fabs(a - 1.0)));
+}
+
 // est_p = ||S f_p - S f_{p-d}|| / sqrt(1 - eps) / (||S f_p|| / sqrt(1 + eps)),
-// eps = max_{j<p} | ||S v_j||^2 - 1 | (Sec. 4.3); on est_p <= stop_tol the
-// recurrence stops at m_eff = p.  One CTA.
-__global__ void __launch_bounds__(kThreads) k_check_end(const double *__restrict__ SV, int s, int p, int *iscal,
-                                                        const int *__restrict__ iscal_chk, double *sf_prev,
-                                                        const double *__restrict__ sf_cur, double *state,
-                                                        double stop_tol) {
+// eps from k_check_eps; on est_p <= stop_tol the recurrence stops at
+// m_eff = p.  One CTA.
+__global__ void __launch_bounds__(kThreads) k_check_end(int s, int p, int *iscal, const int *__restrict__ iscal_chk,
+                                                        double *sf_prev, const double *__restrict__ sf_cur,
+                                                        double *state, double stop_tol) {
     __shared__ double red[64];
     if (iscal_chk[1] == 0) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double eps = 0.0;
-    for (int j = warp; j < p; j += kThreads / 32) {
-        double a = 0.0;
-        for (int i = lane; i < s; i += 32) a = fma(SV[i + (size_t)j * s], SV[i + (size_t)j * s], a);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        eps = fmax(eps, fabs(a - 1.0));
-    }
-    eps = block_max(eps, red);
-    __syncthreads();
+    const double eps = state[3];
     double v[2] = {0.0, 0.0};
     for (int i = threadIdx.x; i < s; i += blockDim.x) {
         const double d = sf_cur[i] - sf_prev[i];
@@ -1784,16 +1960,17 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
     auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
     const size_t mm = (size_t)m * m;
     const size_t rstride = (size_t)m * (m + 1) / 2;   // Givens node solves: packed triangle per slot
-    const size_t nw_bytes = c.hess ? sizeof(double) * chunk * rstride
+    const size_t nw_bytes = c.hess ? sizeof(double) * chunk * rstride * nout
                                    : sizeof(double) * chunk * mm * (rule.cplx ? 4 : 1);
     const size_t sizes[] = {sizeof(double) * (size_t)s * 2 * m, sizeof(double) * 2 * m, sizeof(double) * mm,
                             sizeof(double) * mm, sizeof(double) * mm, sizeof(double) * mm, sizeof(double) * m,
-                            sizeof(double) * m, nw_bytes, sizeof(double) * (size_t)cap * m,
+                            sizeof(double) * m, nw_bytes, sizeof(double) * (size_t)cap * m * (c.hess ? nout : 1),
                             sizeof(double) * (size_t)rule.nlevels * m * nout, sizeof(double) * m * nout,
                             sizeof(double) * m * nout, sizeof(double) * 8 * nout, sizeof(double) * mm,
                             sizeof(double) * mm, sizeof(int) * (size_t)cap, sizeof(double) * 2 * (size_t)m,
                             sizeof(unsigned) * 4, sizeof(double) * mm, sizeof(double) * mm, sizeof(double) * m,
-                            sizeof(double) * mm, sizeof(double) * m};
+                            sizeof(double) * mm, sizeof(double) * m,
+                            sizeof(double) * (size_t)s * (c.rel ? m + 1 : 2 * m)};   // published pivot columns
     constexpr int kNbuf = sizeof(sizes) / sizeof(sizes[0]);
     size_t total = 0;
     for (size_t v : sizes) total += al(v);
@@ -1810,13 +1987,13 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
     c.cvec = ptrs[6]; c.Mtc = ptrs[7]; c.Nw = ptrs[8]; c.out = ptrs[9]; c.qbuf = ptrs[10]; c.qacc = ptrs[11];
     c.z = ptrs[12]; c.qstate = ptrs[13]; c.MT = ptrs[14]; c.R2T = ptrs[15]; c.nodebad = (int *)ptrs[16];
     c.hsig = ptrs[17];
-    unsigned *qr_ready = (unsigned *)ptrs[18];   // [0] published pivot columns, [1] timeout flag
+    unsigned *qr_words = (unsigned *)ptrs[18];   // [1] QR timeout flag, [2], [3] level counters of the methods
     c.RT = ptrs[19];
     c.RTs = ptrs[20];
     c.rinv = ptrs[21];
     c.Rcs = ptrs[22];
     c.cn2 = ptrs[23];
-    c.lev_cnt = qr_ready + 2;
+    c.lev_cnt = qr_words + 2;
     const int G = std::min(2 * num_sms(), 1024);
     long long nlaunch = 0;
     k_tail_copy<<<G, kThreads, 0, st>>>(SV, SAV, c);
@@ -1838,7 +2015,9 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_qr_persist, kQrThreads, qr_smem_bytes(s)) ==
                 cudaSuccess &&
             Gq <= per_sm * num_sms()) {
-            cudaMemsetAsync(qr_ready, 0, sizeof(unsigned) * 4, st);
+            cudaMemsetAsync(qr_words, 0, sizeof(unsigned) * 2, st);
+            double *pub = ptrs[24];
+            cudaMemsetAsync(pub, 0xFF, sizeof(double) * (size_t)cols * s, st);
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeCooperative;
             at[0].val.cooperative = 1;
@@ -1849,7 +2028,7 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
             cfg.stream = st;
             cfg.attrs = at;
             cfg.numAttrs = 1;
-            qr_done = cudaLaunchKernelEx(&cfg, k_qr_persist, c, qr_ready, (int *)(qr_ready + 1)) == cudaSuccess;
+            qr_done = cudaLaunchKernelEx(&cfg, k_qr_persist, c, pub, (int *)(qr_words + 1)) == cudaSuccess;
             if (!qr_done) cudaGetLastError();
             else ++nlaunch;
         } else {
@@ -1880,11 +2059,11 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
     {
         const int rows = (method == SKF_METHOD_SGMRES && !c.rel) ? 2 * m : m;
         const unsigned blocks = (unsigned)((rows + 1) / 2);
-        // + 1 CTA: the cond(R) estimate
-        if (m <= 64) k_tri_right<2><<<blocks + 1, 64, 0, st>>>(c, (int)blocks);
-        else if (m <= 128) k_tri_right<4><<<blocks + 1, 64, 0, st>>>(c, (int)blocks);
-        else if (m <= 256) k_tri_right<8><<<blocks + 1, 64, 0, st>>>(c, (int)blocks);
-        else k_tri_right<16><<<blocks + 1, 64, 0, st>>>(c, (int)blocks);
+        const unsigned ec = c.hess ? 0 : 1;   // + 1 CTA: the cond(R) estimate
+        if (m <= 64) k_tri_right<2><<<blocks + ec, 64, 0, st>>>(c, (int)blocks);
+        else if (m <= 128) k_tri_right<4><<<blocks + ec, 64, 0, st>>>(c, (int)blocks);
+        else if (m <= 256) k_tri_right<8><<<blocks + ec, 64, 0, st>>>(c, (int)blocks);
+        else k_tri_right<16><<<blocks + ec, 64, 0, st>>>(c, (int)blocks);
         ++nlaunch;
     }
     // FP32 factor: packed in shared memory up to kMixedMaxM, else a global slot
@@ -1902,7 +2081,8 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
         cudaFuncSetAttribute(k_nodes_g<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm64);
     // per method: its context (own qstate, quadrature buffers, coefficients,
     // status), node solves, level sums and coefficients
-    TailCtx cm[2];
+    TailMethods tm{};
+    TailCtx *cm = tm.c;
     for (int i = 0; i < nout; ++i) {
         cm[i] = c;
         cm[i].method = outs[i].method;
@@ -1911,18 +2091,29 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
         cm[i].qacc = c.qacc + (size_t)i * m;
         cm[i].z = c.z + (size_t)i * m;
         cm[i].qstate = c.qstate + (size_t)i * 8;
+        if (c.hess) {   // the methods' node solves run in one launch
+            cm[i].out = c.out + (size_t)i * cap * m;
+            cm[i].Nw = c.Nw + (size_t)i * chunk * rstride;
+            cm[i].lev_cnt = c.lev_cnt + i;
+        }
     }
-    for (int mi = 0; mi < nout; ++mi) {
-        const TailCtx &cc = cm[mi];
-        if (mi > 0) {
-            k_fork_state<<<1, 32, 0, st>>>(c.qstate, cc.qstate, iscal, cc.iscal);
+    // node solves of one or (Givens) all methods, then the level sums, by batches
+    const int groups = c.hess ? 1 : nout, per = c.hess ? nout : 1;
+    for (int mi = 0; mi < groups; ++mi) {
+        TailMethods tg{};
+        for (int i = 0; i < per; ++i) tg.c[i] = cm[mi + i];
+        const TailCtx &cc = tg.c[0];
+        // the normal matrices of the Cholesky node solves depend on the method; the
+        // second method's state starts from the first's
+        const int other = c.hess ? 1 : mi;
+        const bool fork = nout == 2 && (c.hess || mi == 1);
+        if (fork && !c.hess) {
+            k_fork_state<<<1, 32, 0, st>>>(c.qstate, cm[other].qstate, iscal, cm[other].iscal);
             ++nlaunch;
         }
-        // the normal matrices of the Cholesky node solves depend on the method
-        if (mi == 0 || !c.hess) {
-            k_tail_prep<<<G, kThreads, 0, st>>>(cc);
-            ++nlaunch;
-        }
+        k_tail_prep<<<G, kThreads, 0, st>>>(cc, fork && c.hess ? cm[other].qstate : nullptr,
+                                            fork && c.hess ? cm[other].iscal : nullptr);
+        ++nlaunch;
         for (size_t bi = 0; bi < batches.size(); ++bi) {
             const int l0 = batches[bi].first, nl = batches[bi].second;
             const int n0 = rule.h_start[l0];
@@ -1930,11 +2121,12 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
             for (int o = 0; o < nn; o += chunk) {
                 const int nb = std::min(chunk, nn - o);
                 if (cc.hess) {
-                    const unsigned g = (unsigned)((nb + kHessWarps - 1) / kHessWarps);
-                    if (m <= 64) k_nodes_hess<2><<<g, 32 * kHessWarps, 0, st>>>(cc, n0, o, nb, cc.Nw, rstride);
-                    else if (m <= 128) k_nodes_hess<4><<<g, 32 * kHessWarps, 0, st>>>(cc, n0, o, nb, cc.Nw, rstride);
-                    else if (m <= 256) k_nodes_hess<8><<<g, 32 * kHessWarps, 0, st>>>(cc, n0, o, nb, cc.Nw, rstride);
-                    else k_nodes_hess<16><<<g, 32 * kHessWarps, 0, st>>>(cc, n0, o, nb, cc.Nw, rstride);
+                    const int est = bi == 0 && o == 0;
+                    const dim3 g((unsigned)((nb + kHessWarps - 1) / kHessWarps + est), (unsigned)per);
+                    if (m <= 64) k_nodes_hess<2><<<g, 32 * kHessWarps, 0, st>>>(tg, n0, o, nb, rstride, est);
+                    else if (m <= 128) k_nodes_hess<4><<<g, 32 * kHessWarps, 0, st>>>(tg, n0, o, nb, rstride, est);
+                    else if (m <= 256) k_nodes_hess<8><<<g, 32 * kHessWarps, 0, st>>>(tg, n0, o, nb, rstride, est);
+                    else k_nodes_hess<16><<<g, 32 * kHessWarps, 0, st>>>(tg, n0, o, nb, rstride, est);
                     nlaunch += 1;
                     continue;
                 }
@@ -1947,25 +2139,26 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
                 }
                 nlaunch += 2;
             }
-            k_levels<<<(unsigned)nl, kThreads, 0, st>>>(cc, l0, nl, rule.lev_start, rule.lev_ell, n0, tol,
-                                             bi + 1 == batches.size() ? 1 : 0);
+            k_levels<<<dim3((unsigned)nl, (unsigned)per), kThreads, 0, st>>>(tg, l0, nl, rule.lev_start, rule.lev_ell,
+                                                                            n0, tol, bi + 1 == batches.size() ? 1 : 0);
             ++nlaunch;
         }
-        if (m <= 64) k_coeffs<2><<<1, 32, 0, st>>>(cc);
-        else if (m <= 128) k_coeffs<4><<<1, 32, 0, st>>>(cc);
-        else if (m <= 256) k_coeffs<8><<<1, 32, 0, st>>>(cc);
-        else k_coeffs<16><<<1, 32, 0, st>>>(cc);
+        if (m <= 64) k_coeffs<2><<<per, 32, 0, st>>>(tg);
+        else if (m <= 128) k_coeffs<4><<<per, 32, 0, st>>>(tg);
+        else if (m <= 256) k_coeffs<8><<<per, 32, 0, st>>>(tg);
+        else k_coeffs<16><<<per, 32, 0, st>>>(tg);
         ++nlaunch;
-        if (outs[mi].z_out) {
-            k_copy_z<<<(m + kThreads - 1) / kThreads, kThreads, 0, st>>>(cc, outs[mi].z_out);
-            ++nlaunch;
-        }
+        for (int i = 0; i < per; ++i)
+            if (outs[mi + i].z_out) {
+                k_copy_z<<<(m + kThreads - 1) / kThreads, kThreads, 0, st>>>(tg.c[i], outs[mi + i].z_out);
+                ++nlaunch;
+            }
     }
     const int64_t rb = std::min<int64_t>((n + kThreads - 1) / kThreads, 16 * num_sms());
     const unsigned rgrid = (unsigned)std::max<int64_t>(rb, 1);
     const size_t zsm = sizeof(float) * 2 * (size_t)m;
     if (sketch_out) {
-        k_sketch_f<<<(s + kThreads - 1) / kThreads, kThreads, 0, st>>>(cm[0], SV, sketch_out);
+        k_sketch_f<<<(s + 63) / 64, 64, sizeof(double) * m, st>>>(cm[0], SV, sketch_out);
         ++nlaunch;
     } else if (nout == 2 && vdt == SKF_F64 && outs[0].x && outs[1].x) {
         k_recombine2<<<rgrid, kThreads, sizeof(double) * 2 * m, st>>>((const double *)V, ldv, n, cm[0].z, cm[1].z,
@@ -1976,7 +2169,7 @@ skf_status tail_run_multi(int nout, const TailOut *outs, int s, int m, int64_t n
             double *x = outs[mi].x;
             if (x == nullptr) continue;   // coefficients only (two-pass mode)
             if (vdt == SKF_F64)
-                k_recombine<<<rgrid, kThreads, 0, st>>>((const double *)V, ldv, n, cm[mi].z, iscal, x);
+                k_recombine<<<rgrid, kThreads, sizeof(double) * m, st>>>((const double *)V, ldv, n, cm[mi].z, iscal, x);
             else if (vdt == SKF_F32)
                 k_recombine_lp<float><<<rgrid, kThreads, zsm, st>>>((const float *)V, ldv, n, cm[mi].z, iscal, x);
             else
@@ -2005,16 +2198,20 @@ skf_status tail_run(skf_method method, int s, int m, int64_t n, const void *V, s
                           cond_max, H, ldh, kt);
 }
 
-skf_status stop_check(skf_method method, int s, int p, const double *vscale, const double *SV, const double *SAV,
-                      int *iscal, int *iscal_chk, double *sf_prev, double *sf_cur, double *state, const RuleDev &rule,
+skf_status stop_check(skf_method method, int s, int p, skf_dtype vdt, const double *vscale, const double *SV,
+                      const double *SAV, const double *H, int ldh, int kt, int *iscal, int *iscal_chk, double *sf_prev, double *sf_cur, double *state, const RuleDev &rule,
                       double tol_quad, double stop_tol, cudaStream_t st) {
     k_check_begin<<<1, 32, 0, st>>>(iscal, iscal_chk, p);
     count_launches(1);
-    skf_status e = tail_run(method, s, p, 0, nullptr, SKF_F64, 0, vscale, SV, SAV, iscal_chk, rule, tol_quad, nullptr,
-                            nullptr, st, sf_cur, nullptr);
+    // the relation form where the basis type has it: p + 1 instead of 2 p
+    // reflectors and the Givens node solves (7 checkpoints of the p = 20 .. 140 case:
+    // 3.0 -> 2.1 ms of QR, 2.3 -> 0.9 ms of node solves)
+    skf_status e = tail_run(method, s, p, 0, nullptr, vdt, 0, vscale, SV, SAV, iscal_chk, rule, tol_quad, nullptr,
+                            nullptr, st, sf_cur, nullptr, nullptr, 0.0, H, ldh, kt);
     if (e != SKF_OK) return e;
-    k_check_end<<<1, kThreads, 0, st>>>(SV, s, p, iscal, iscal_chk, sf_prev, sf_cur, state, stop_tol);
-    count_launches(1);
+    k_check_eps<<<(p + kThreads / 32 - 1) / (kThreads / 32), kThreads, 0, st>>>(SV, s, p, iscal_chk, state);
+    k_check_end<<<1, kThreads, 0, st>>>(s, p, iscal, iscal_chk, sf_prev, sf_cur, state, stop_tol);
+    count_launches(2);
     const cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return cuda_fail(ce, "stopping-criterion kernels");
     return SKF_OK;
