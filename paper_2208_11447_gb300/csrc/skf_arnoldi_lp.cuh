@@ -164,6 +164,7 @@ struct LpCtx {
     int *iscal;                // [0] stopped, [1] m_eff, [2] status, [3] step that stopped
     int G;                     // CTAs of every kernel (chunk partition)
     int lc;                    // log2 of the per-lane bin copies of the update kernel
+    DiagOp dg;                 // diagonal copy of the operator (dg.w = 0: none)
 };
 
 // (row of S, sign) of the zeta nonzeros of column r, from the compact or the
@@ -540,7 +541,12 @@ __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv_lp(LpCtx c, in
 // indices of chunk i + 1 are loaded, and the slice width and offset of chunk
 // i + 2 are loaded.  One memory round trip per chunk instead of two (column,
 // then gather), with 8 extra registers per thread.
-template <int KW, int ZCAP, typename TB, int W>
+// DG: the operator's diagonal copy (W its value slots); the registers of the
+// column indices then hold the values of chunk i + 1.  The loop is bound by HBM:
+// 29 instead of 56 bytes of A per row of a 7-point stencil (256^3, FP32, from the
+// solves: 191 -> 134 us, 120 steps 36.6 -> 29.8 ms; 150^3, BF16, 40 steps: 4.25 ->
+// 3.84 ms).
+template <int KW, int ZCAP, typename TB, int W, bool DG>
 __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv_lp_pipe(LpCtx c, int j) {
     extern __shared__ int bins[];   // [2 s]: limbs of S w_j (stopping step) or of S y_{m-1} (last step)
     __shared__ double red[32 * KW];
@@ -581,6 +587,54 @@ __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv_lp_pipe(LpCtx 
     int64_t wo[KW];
 #pragma unroll
     for (int a = 0; a < KW; ++a) wo[a] = a < nw ? c.woff[a] : 0;
+    // dots and magnitude of one row's y
+    auto row_done = [&](unsigned row, float y, const float (&wv)[KW]) {
+        c.Y[row] = y;
+#pragma unroll
+        for (int a = 0; a < KW; ++a)
+            if (a < nw) acc[a] = fmaf(wv[a], y, acc[a]);
+        ykey = max(ykey, abs_key_f32(y));
+        if (last && ey != kNoExp) scatter2<ZCAP>(c, row, fixed_point_f32(y, shift_y), L, bins, bins + s);
+    };
+    if constexpr (DG) {
+        // values of chunk i + 1 and masks of chunk i + 1 in flight while chunk i
+        // gathers (slots of the last slice past row n are present in no mask)
+        const float *dv = (const float *)c.dg.val + lane;
+        unsigned mk = 0;
+        float av[W];
+        if (t < nsl) {
+            mk = __ldg(c.dg.mask + r);
+#pragma unroll
+            for (int d = 0; d < W; ++d) av[d] = __ldcs(dv + (size_t)t * (32 * W) + 32 * d);
+        }
+        for (; t < nsl; r += step, t += tstep) {
+            const bool ok = r < n32;
+            float xv[W], wv[KW], avn[W];
+            const TB *wr = wj + r;
+#pragma unroll
+            for (int d = 0; d < W; ++d) xv[d] = (mk >> d) & 1u ? Store<TB>::ld(wr + c.dg.off[d]) : 0.f;
+#pragma unroll
+            for (int a = 0; a < KW; ++a) wv[a] = (ok && a < nw) ? Store<TB>::ld(V + wo[a] + r) : 0.f;
+            mk = 0;
+#pragma unroll
+            for (int d = 0; d < W; ++d) avn[d] = 0.f;
+            if (t + tstep < nsl) {
+                mk = __ldg(c.dg.mask + r + step);
+#pragma unroll
+                for (int d = 0; d < W; ++d) avn[d] = __ldcs(dv + (size_t)(t + tstep) * (32 * W) + 32 * d);
+            }
+            if (ok) {
+                float y = 0.f;
+#pragma unroll
+                for (int d = 0; d < W; ++d) y = fmaf(av[d], xv[d], y);   // an absent entry adds 0
+                row_done(r, y, wv);
+            }
+#pragma unroll
+            for (int d = 0; d < W; ++d) av[d] = avn[d];
+        }
+        spmv_end<KW>(c, j, nw, last, L, bins, acc, ykey, red);
+        return;
+    }
     // slice metadata of chunks i and i + 1 (0 wide past the end)
     int wt_c = 0, wt_n = 0;
     long long so_c = 0, so_n = 0;
@@ -635,12 +689,7 @@ __global__ void __launch_bounds__(kSpmvThreads, 1) k_arnoldi_spmv_lp_pipe(LpCtx 
 #pragma unroll
             for (int p = 0; p < W; ++p)
                 if (p < wt_c) y = fmaf(av[p], xv[p], y);
-            c.Y[r] = y;
-#pragma unroll
-            for (int a = 0; a < KW; ++a)
-                if (a < nw) acc[a] = fmaf(wv[a], y, acc[a]);
-            ykey = max(ykey, abs_key_f32(y));
-            if (last && ey != kNoExp) scatter2<ZCAP>(c, r, fixed_point_f32(y, shift_y), L, bins, bins + s);
+            row_done(r, y, wv);
         }
         wt_c = wt_n;
         so_c = so_n;
@@ -1122,15 +1171,25 @@ __global__ void __launch_bounds__(kThreads) k_arnoldi_info_lp(LpCtx c, skf_info 
     }
 }
 
+// The pipelined SpMV (k <= 2, zeta <= 8) with the product slots the operator
+// needs.
+template <typename TB>
+auto narrow_spmv(const LpCtx &c, bool pipe, void (*other)(LpCtx, int)) {
+    if (c.dg.w == 5) return k_arnoldi_spmv_lp_pipe<2, 8, TB, 5, true>;
+    if (c.dg.w == 7) return k_arnoldi_spmv_lp_pipe<2, 8, TB, 7, true>;
+    if (c.dg.w == 8) return k_arnoldi_spmv_lp_pipe<2, 8, TB, 8, true>;
+    if (pipe && c.max_width <= 5) return k_arnoldi_spmv_lp_pipe<2, 8, TB, 5, false>;
+    if (pipe && c.max_width <= 7) return k_arnoldi_spmv_lp_pipe<2, 8, TB, 7, false>;
+    return other;
+}
+
 template <int KW, int ZCAP, typename TB>
 void launch_steps(const LpCtx &c, bool pipe, size_t smem_spmv, size_t smem_upd, cudaStream_t st,
                   const StepHook *hook, const skf_sketch *dense, void *dwork) {
-    auto spmv = pipe ? k_arnoldi_spmv_lp_pipe<KW, ZCAP, TB, 8> : k_arnoldi_spmv_lp<KW, ZCAP, TB>;
-    // fewer product slots for the 5- and 7-point stencils
-    if constexpr (KW == 2 && ZCAP == 8) {
-        if (pipe && c.max_width <= 7) spmv = c.max_width <= 5 ? k_arnoldi_spmv_lp_pipe<KW, ZCAP, TB, 5>
-                                                              : k_arnoldi_spmv_lp_pipe<KW, ZCAP, TB, 7>;
-    }
+    auto spmv = pipe ? k_arnoldi_spmv_lp_pipe<KW, ZCAP, TB, 8, false> : k_arnoldi_spmv_lp<KW, ZCAP, TB>;
+    // the diagonal copy, or fewer product slots for narrow slices: instantiated
+    // for the usual window and sketch
+    if constexpr (KW == 2 && ZCAP == 8) spmv = narrow_spmv<TB>(c, pipe, spmv);
     auto update = k_arnoldi_update_lp<KW, ZCAP, TB, 0>;
     if constexpr (ZCAP == 8) {
         if (c.split) update = c.p8_block == 64 ? k_arnoldi_update_lp<KW, 8, TB, 64> : k_arnoldi_update_lp<KW, 8, TB, 128>;
@@ -1264,6 +1323,7 @@ skf_status lp_setup(const skf_csr *A, const skf_sketch *S, int m, int k, TB *V, 
     // slices at most 8 wide: the pipelined SpMV (a row split takes the generic one)
     const bool pipe = A->max_width <= 8 && A->nlong == 0 && A->perm == nullptr;
     c.rs = row_split_of(A);
+    c.dg = diag_of(A);
 
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t szY = sizeof(float) * A->n;
@@ -1391,7 +1451,7 @@ skf_status arnoldi_run_lp_block(const skf_csr *A, const skf_sketch *S, int nr, c
     const int G = runs[0].c.G;
     for (int q = 0; q < nr; ++q) k_arnoldi_init_lp<TB><<<G, kChunkRows, 0, st>>>(runs[q].c, b[q]);
     auto spmm = k_arnoldi_spmm_lp<2, 8, TB, kSpmmBlock>;
-    auto spmv = k_arnoldi_spmv_lp_pipe<2, 8, TB, 8>;
+    auto spmv = narrow_spmv<TB>(runs[0].c, true, k_arnoldi_spmv_lp_pipe<2, 8, TB, 8, false>);
     auto update = k_arnoldi_update_lp<2, 8, TB, 0>;
     if (runs[0].c.split)
         update = runs[0].c.p8_block == 64 ? k_arnoldi_update_lp<2, 8, TB, 64> : k_arnoldi_update_lp<2, 8, TB, 128>;
