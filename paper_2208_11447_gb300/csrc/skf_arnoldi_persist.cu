@@ -34,10 +34,8 @@
 // roundoff of ||A v_j||).  The last column (and the column at a happy
 // breakdown, where no further vector is formed) is sketched directly.
 //
-// Cross-CTA sums: per-CTA partials of the dots in global memory, reduced
-// after the barrier by every CTA in the same fixed order (deterministic);
-// integer sketch partials added with 64-bit global atomics (exact, so the
-// order does not matter).  Every barrier wait is bounded by a clock64
+// Cross-CTA sums: exact integer sums of the dots and sketch partials, added
+// with 64-bit global atomics (the order does not matter; see push_sums).  Every barrier wait is bounded by a clock64
 // budget: past it the kernel records SKF_ERR_TIMEOUT, and every CTA returns
 // at its next barrier.
 #include <math.h>
@@ -66,6 +64,7 @@ struct PCtx {
     const int32_t *sell_w;
     const void *sell_val;      // T values (T = double, or float for an FP32 basis)
     const int32_t *sell_col;
+    DiagOp dg;                 // diagonal copy of the operator (dg.w = W, or 0: none)
     float l2_frac;             // share of the operator's lines kept in L2 from step to step
     SparseSign sp;
     const uint16_t *pattern;   // [n][zeta]
@@ -417,7 +416,8 @@ constexpr int kSpmvWarps = kPNW - 1;   // the last warp serves the reductions
 template <int KW, int W, typename T>
 __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ wsrc, const T *win,
                                           const int (&soff)[KW], int nw, T *ys, const long long *meta_o,
-                                          const int *meta_w, int nsl, int nr, T (&acc)[KW], unsigned &ykey) {
+                                          const int *meta_w, uint2 dmask, int nsl, int nr, T (&acc)[KW],
+                                          unsigned &ykey) {
     const T *sell_val = (const T *)c.sell_val;
     const unsigned long long pol = operator_policy(c.l2_frac);
     const int lane = threadIdx.x & 31;
@@ -427,6 +427,52 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
         next_t += kSpmvWarps;
         return t;
     };
+    if (W > 0 && c.dg.w != 0) {
+        // diagonal copy: values and gathers of slice tn and the masks of slice
+        // tnn in flight while slice t is computed (a row past nr is present in no
+        // mask); the first two masks are the same in every step (dmask), so the
+        // gathers start with the phase.  Per step, slices / this copy: 100^3 grid
+        // FP64 37.0 / 34.5 us, FP32 25.1 / 23.6; 25600 rows 9.8 / 9.6; 10^4 rows
+        // 9.9 / 10.0.  (A guard around the whole load instead of one per value: 35.8
+        // and 25.2 us.)
+        constexpr int WD = W > 0 ? W : 1;
+        const int64_t r0 = (int64_t)blockIdx.x * c.R;
+        const T *dv = (const T *)c.dg.val + r0 * W + lane;
+        const T *wr = wsrc + r0 + lane;
+        const uint8_t *mk = c.dg.mask + r0 + lane;
+        struct Stage {
+            T av[WD], xv[WD];
+        };
+        auto load = [&](int t, unsigned m, Stage &q) {
+#pragma unroll
+            for (int d = 0; d < W; ++d) {
+                q.av[d] = t < nsl ? ld_op(dv + t * (32 * W) + 32 * d, pol) : T(0);
+                q.xv[d] = (m >> d) & 1u ? __ldcg(wr + 32 * t + c.dg.off[d]) : T(0);
+            }
+        };
+        auto mask_of = [&](int t) { return t < nsl ? (unsigned)__ldg(mk + 32 * t) : 0u; };
+        Stage cur, nxt;
+        int t = next_t;
+        load(t, dmask.x, cur);
+        unsigned mn = dmask.y;
+        for (; t < nsl; t += kSpmvWarps) {
+            load(t + kSpmvWarps, mn, nxt);
+            mn = mask_of(t + 2 * kSpmvWarps);
+            const int lr = t * 32 + lane;
+            if (lr < nr) {
+                T y = T(0);
+#pragma unroll
+                for (int d = 0; d < W; ++d) y = fma(cur.av[d], cur.xv[d], y);   // an absent entry adds 0
+                ys[lr] = y;
+#pragma unroll
+                for (int a = 0; a < KW; ++a)
+                    if (a < nw) acc[a] = fma(win[soff[a] + lr], y, acc[a]);
+                ykey = max(ykey, mag_key(y));
+            }
+            cur = nxt;
+        }
+        return;
+    }
     if constexpr (W > 0) {
         // three-stage pipeline: values and gathers of slice tn and column
         // indices of slice tnn are in flight while slice t is computed
@@ -649,6 +695,11 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
         meta_o[t] = c.sell_off[r0 / 32 + t];
         meta_w[t] = c.sell_w[r0 / 32 + t];
     }
+    uint2 dmask = make_uint2(0u, 0u);   // masks of this warp's first two slices (diagonal copy)
+    if (W > 0 && c.dg.w != 0 && warp < kSpmvWarps) {
+        if (warp < nsl) dmask.x = c.dg.mask[r0 + 32 * warp + lane];
+        if (warp + kSpmvWarps < nsl) dmask.y = c.dg.mask[r0 + 32 * (warp + kSpmvWarps) + lane];
+    }
     for (int i = tid; i < 4 * nbin; i += kPT) bins[i] = 0;
     for (int64_t i = (int64_t)g * kPT + tid; i < (int64_t)(m + 1) * m; i += (int64_t)G * kPT) c.H[i] = 0.0;
     if (g == 0 && tid == 0) {
@@ -782,7 +833,8 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
 #pragma unroll
             for (int a = 0; a < KW; ++a) soff[a] = a < nw ? ((i0 + a) % k) * R : 0;
             if (warp < kSpmvWarps)
-                spmv_rows<KW, W, T>(c, Vb + (size_t)j * c.ldv, win, soff, nw, ys, meta_o, meta_w, nsl, nr, acc, ykey);
+                spmv_rows<KW, W, T>(c, Vb + (size_t)j * c.ldv, win, soff, nw, ys, meta_o, meta_w, dmask, nsl, nr, acc,
+                                    ykey);
         }
         if (flush_all && j >= 1) flush_w(j - 1, tid, kPT);
         __syncthreads();   // the bounds ea[] of the service warp
@@ -849,7 +901,8 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             for (int a = 0; a < KW; ++a) accb[a] = T(0);
             unsigned kb = 0;
             if (warp < kSpmvWarps)
-                spmv_rows<KW, W, T>(c, Vb + (size_t)jb * c.ldv, win, soff, 0, ys, meta_o, meta_w, nsl, nr, accb, kb);
+                spmv_rows<KW, W, T>(c, Vb + (size_t)jb * c.ldv, win, soff, 0, ys, meta_o, meta_w, dmask, nsl, nr, accb,
+                                    kb);
             __syncthreads();
             const int ey = eys[jb & 3];
             const int shift_y = c.frac - (ey == kNoExp ? 0 : ey);
@@ -1134,13 +1187,16 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     c.sell_w = A->sell_w;
     c.sell_val = A->sell_val;
     c.sell_col = A->sell_col;
+    // 8 diagonals of rows at most 7 wide: only the general FP64 form has 8 slots
+    if (A->dia_w <= (f32 || yg ? 7 : 8)) c.dg = diag_of(A);
     // L2 share of the operator, measured per step (keep none / this rule): all of
     // it up to 90 MB (FP64 41.9 / 41.1 us at 84 MB, 21.6 / 20.2 at 22 MB; FP32
     // 32.8 / 26.4 at 56 MB), beyond that 50 MB of it (FP32 47.8 / 45.2 at 97 MB;
     // all of it 48.5).  With y~ in global memory L2 already holds that and the
     // gathered vector, and a kept operator only displaces them (FP64 50.2 / 53.2
     // at 106 MB, 49.3 / 52.9 at 84 MB): nothing is kept.
-    const double opb = (double)A->sell_entries * (double)(vb + 4);
+    const double opb = c.dg.w != 0 ? 32.0 * (double)A->nslices * (double)(vb * c.dg.w + 1)
+                                   : (double)A->sell_entries * (double)(vb + 4);
     c.l2_frac = yg ? 0.f : opb <= 90e6 ? 1.f : (float)(50e6 / opb);
     c.sp = make_sparse_sign(S);
     c.pattern = S->pattern;
@@ -1195,10 +1251,11 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     cudaMemsetAsync(c.slot, 0, (size_t)((char *)c.Sw - (char *)c.slot), st);
     cudaMemsetAsync(c.bar, 0, szBar, st);
     cudaError_t e;
-    if (f32) e = launch_persist_f32(c, A->max_width, G, smem, st);
-    else if (yg) e = launch_persist_yg(c, A->max_width, G, smem, st);
-    else if (KW == 2) e = launch_persist_w<2>(c, A->max_width, G, smem, st);
-    else e = launch_persist_w<4>(c, A->max_width, G, smem, st);
+    const int slots = c.dg.w != 0 ? c.dg.w : A->max_width;   // product slots of the kernel
+    if (f32) e = launch_persist_f32(c, slots, G, smem, st);
+    else if (yg) e = launch_persist_yg(c, slots, G, smem, st);
+    else if (KW == 2) e = launch_persist_w<2>(c, slots, G, smem, st);
+    else e = launch_persist_w<4>(c, slots, G, smem, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         dfree(ws, st);
