@@ -870,7 +870,7 @@ __device__ __forceinline__ int sum_copies(const int *b, int i, int lc) {
 }
 
 // Per-lane bin copies of the split layout: 2 * SB * 8 bins per limb, C copies,
-// 64 KB per limb either way.
+// 64 KB per limb either way; the two limbs of w_j are paired (scatter8_paired).
 template <int SB> struct SplitGeom {
     static constexpr int kLc = SB == 64 ? 4 : 3;
     static constexpr int kBins = 8 * 2 * SB;
@@ -971,9 +971,9 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_arnoldi_update_lp(LpCtx c, i
     // Row loop.  This kernel is bound by instruction issue (IPC 2.6 to 3.1 of 4
     // with 64-bit row arithmetic and a bin address per atomic), so rows are
     // 32-bit, the window coefficients stay in registers and the compact pattern
-    // takes four instructions per nonzero (scatter8).  The loads of the next
+    // takes immediate bin offsets (scatter8_paired).  The loads of the next
     // U chunks are issued before the arithmetic of these.  N = 16.8M, FP32:
-    // 114 -> 93 us; BF16, N = 3.4M: 60 -> 47 us.  The rows a thread adds up,
+    // 114 -> 93 us (79 with the paired limbs); BF16, N = 3.4M: 60 -> 47 us.  The rows a thread adds up,
     // and their order, do not depend on U.
     constexpr int U = KW <= 2 ? 2 : 1;       // chunks per iteration and thread
     constexpr bool kAhead = KW <= 4;         // wider windows do not fit in the registers twice
@@ -1002,7 +1002,8 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_arnoldi_update_lp(LpCtx c, i
         }
     };
     // shared-memory addresses of this lane's bin copies (split layout)
-    const unsigned wbase = shared_address(wb0) + 4u * (unsigned)(lane & cm);
+    constexpr int kLc = split ? SplitGeom<SB ? SB : 64>::kLc : 0;
+    const PairedLane<kLc> pl(wb0, lane);
     const unsigned dbase = shared_address(db) + 4u * (unsigned)(lane & cm);
     Rows cur, nxt;
     unsigned rb = blockIdx.x * kChunkRows + threadIdx.x;
@@ -1024,7 +1025,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_arnoldi_update_lp(LpCtx c, i
                 int l0, l1;
                 limbs_f32(wv[0], lsw, l0, l1);
                 if constexpr (split) {
-                    scatter8<SB, SplitGeom<SB>::kLc>(cur.pv[u], wbase, l0, l1);
+                    scatter8_paired<SB, kLc>(cur.pv[u], pl.a1, pl.a2, pl.swap ? l1 : l0, pl.swap ? l0 : l1);
                 } else {
 #pragma unroll
                     for (int q = 0; q < ZCAP; ++q)
@@ -1074,8 +1075,10 @@ __global__ void __launch_bounds__(kUpdThreads, 1) k_arnoldi_update_lp(LpCtx c, i
                 int q = 0;
                 while (q + 1 < 8 && i >= c.sp.start[q + 1]) ++q;
                 const int bp = 2 * SB * q + (i - c.sp.start[q]), bn = bp + SB;   // positive and negative bins
-                v0 = (long long)sum_copies(wb0, bp, lc) - sum_copies(wb0, bn, lc);
-                v1 = (long long)sum_copies(wb1, bp, lc) - sum_copies(wb1, bn, lc);
+                int s0, s1;
+                paired_sums<kLc>(wb0, bp, bn, s0, s1);
+                v0 = s0;
+                v1 = s1;
                 if (resid) vd = (long long)sum_copies(db, bp, lc) - sum_copies(db, bn, lc);
             } else {
                 v0 = sum_copies(wb0, i, lc);

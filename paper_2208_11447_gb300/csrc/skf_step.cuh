@@ -89,6 +89,23 @@ __device__ __forceinline__ void scatter8(uint2 pv, unsigned base, int l0, int l1
         scatter8<BLK, LC, Q + 1>(pv, base, l0, l1);
     }
 }
+// The same with the copies of both limbs side by side: a bin is 2 << LC words
+// [limb][copy], and of two lanes that share a copy of their limb's words one
+// adds limb 0 first and the other limb 1 (a1, v1 first, then a2, v2: see
+// PairedLane).  With LC = 4 a warp's 32 adds fall into 32 banks whatever the
+// rows; with the limbs in separate arrays two lanes shared each bank (reduced-
+// precision update at N = 16.8M, from the solves: 87 -> 79 us).  One instruction
+// more per nonzero: with fewer copies, where lanes still collide, it is the slower
+// form (sketch apply, 4 copies: 226 -> 280 us).
+template <int BLK, int LC, int Q = 0>
+__device__ __forceinline__ void scatter8_paired(uint2 pv, unsigned a1, unsigned a2, int v1, int v2) {
+    if constexpr (Q < 8) {
+        const unsigned e = __byte_perm(Q < 4 ? pv.x : pv.y, 0u, 0x4440u + (Q & 3)) << (LC + 3);
+        red_shared<(Q * 2 * BLK) << (LC + 3)>(a1 + e, v1);
+        red_shared<(Q * 2 * BLK) << (LC + 3)>(a2 + e, v2);
+        scatter8_paired<BLK, LC, Q + 1>(pv, a1, a2, v1, v2);
+    }
+}
 // one limb only
 template <int BLK, int LC, int Q = 0>
 __device__ __forceinline__ void scatter8_one(uint2 pv, unsigned base, int l0) {
@@ -99,6 +116,30 @@ __device__ __forceinline__ void scatter8_one(uint2 pv, unsigned base, int l0) {
     }
 }
 __device__ __forceinline__ unsigned shared_address(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+// A lane's place in paired bins of 1 << LC copies.
+template <int LC> struct PairedLane {
+    unsigned a1, a2;
+    bool swap;   // limb 1 first
+    __device__ __forceinline__ PairedLane(const void *bins, int lane) {
+        constexpr unsigned C = 1u << LC;
+        swap = ((unsigned)lane & C) != 0u;
+        const unsigned a = shared_address(bins) + 4u * ((unsigned)lane & (C - 1u));
+        a1 = a + (swap ? 4u * C : 0u);
+        a2 = a + (swap ? 0u : 4u * C);
+    }
+};
+// Limb sums (positive minus negative bin) of a row of S from paired bins, by one
+// warp; exact in 32 bits, since all contributions of the row fit together.
+template <int LC>
+__device__ __forceinline__ void paired_sums(const int *bins, int pos, int neg, int &v0, int &v1) {
+    constexpr int C = 1 << LC;
+    const int lane = threadIdx.x & 31;
+    int v = lane < 2 * C ? bins[(pos << (LC + 1)) + lane] - bins[(neg << (LC + 1)) + lane] : 0;
+#pragma unroll
+    for (int o = C / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    v0 = __shfl_sync(0xffffffffu, v, 0);
+    v1 = __shfl_sync(0xffffffffu, v, C);
+}
 
 // Arrival ticket: true in exactly one CTA, the last to finish its partials.
 __device__ __forceinline__ bool last_to_arrive(unsigned *cnt) {
