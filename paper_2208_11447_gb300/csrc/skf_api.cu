@@ -947,8 +947,13 @@ static void free_layout(skf_csr *A) {
 // up to 5, 7 or 8, the instantiations of the step kernels; the unused ones
 // repeat the last diagonal and are absent in every row.  An operator it does
 // not fit, or for which there is no memory left, keeps the slices alone.
+// Small operators keep the slices: they live in L2 and a step is latency (10^4 rows:
+// 9.9 us per step with the slices, 10.0 with the copy; 25600 rows: 9.8 and 9.6), while
+// the copy's launches and allocation add 0.3 ms to the upload.
+constexpr int64_t kDiagMinRows = 16384;
 static skf_status build_diagonals(skf_csr *A, cudaStream_t st) {
     const size_t esz = A->vdtype == SKF_F64 ? 8 : 4;
+    if (A->n < kDiagMinRows) return SKF_OK;
     if (A->perm != nullptr || A->nlong > 0 || A->max_width > 8 || A->nnz == 0) return SKF_OK;
     int *tab = nullptr, h[9];
     if (dalloc((void **)&tab, sizeof(h), st) != SKF_OK) return SKF_OK;
@@ -985,10 +990,8 @@ static skf_status build_diagonals(skf_csr *A, cudaStream_t st) {
         k_diag_fill<<<blocks, 256, 0, st>>>(A->rowptr, A->colind, (const float *)A->values, A->n, A->nslices, off, w,
                                             (float *)A->dia_val, A->dia_mask);
     count_launches(1);
-    e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "diagonal fill");
     A->dia_w = w;
-    return SKF_OK;
+    return SKF_OK;   // (the caller synchronises)
 }
 
 static skf_status build_layout(skf_csr *A, int cut, int sort, cudaStream_t st) {
@@ -1008,8 +1011,11 @@ static skf_status build_layout(skf_csr *A, int cut, int sort, cudaStream_t st) {
         const int32_t len = hrp[r + 1] - hrp[r];
         return len > cut ? 0 : len;
     };
-    std::vector<int32_t> hperm((size_t)n);
-    for (int64_t i = 0; i < n; ++i) hperm[i] = (int32_t)i;
+    std::vector<int32_t> hperm;   // slot -> row of a sorted layout (the slots are the rows otherwise)
+    if (sort != 0) {
+        hperm.resize((size_t)n);
+        for (int64_t i = 0; i < n; ++i) hperm[i] = (int32_t)i;
+    }
     auto padded_of = [&]() {
         int64_t pad = 0;
         for (int64_t t = 0; t < A->nslices; ++t) {
@@ -1028,12 +1034,17 @@ static skf_status build_layout(skf_csr *A, int cut, int sort, cudaStream_t st) {
                              [&](int32_t x, int32_t y) { return eff(x) > eff(y); });
         }
         sorted = sort == 1 || padded_of() * 5 < pad_plain * 4;
-        if (!sorted)
-            for (int64_t i = 0; i < n; ++i) hperm[i] = (int32_t)i;
     }
+    auto row_at = [&](int64_t i) { return sorted ? (int64_t)hperm[i] : i; };
+    bool any_long = false;
     for (int64_t t = 0; t < A->nslices; ++t) {
         int mx = 0;
-        for (int64_t i = 32 * t; i < std::min<int64_t>(n, 32 * t + 32); ++i) mx = std::max(mx, eff(hperm[i]));
+        for (int64_t i = 32 * t; i < std::min<int64_t>(n, 32 * t + 32); ++i) {
+            const int64_t r = row_at(i);
+            const int32_t len = hrp[r + 1] - hrp[r];
+            any_long |= len > cut;
+            mx = std::max(mx, len > cut ? 0 : len);
+        }
         hw[t] = mx;
     }
     if (sorted) {
@@ -1045,13 +1056,13 @@ static skf_status build_layout(skf_csr *A, int cut, int sort, cudaStream_t st) {
     }
     cudaMemcpyAsync(A->sell_w, hw.data(), sizeof(int32_t) * A->nslices, cudaMemcpyHostToDevice, st);
     // row split: long rows, their segments and the per-slice masks
-    std::vector<uint2> hl((size_t)A->nslices, make_uint2(0u, 0u));
+    std::vector<uint2> hl(any_long ? (size_t)A->nslices : 0, make_uint2(0u, 0u));
     std::vector<int32_t> seg0{0}, sb, se;
     int64_t nl = 0;
-    for (int64_t t = 0; t < A->nslices; ++t) {
+    for (int64_t t = 0; any_long && t < A->nslices; ++t) {
         hl[t].y = (unsigned)nl;
         for (int l = 0; l < 32 && 32 * t + l < n; ++l) {
-            const int64_t r = hperm[32 * t + l];
+            const int64_t r = row_at(32 * t + l);
             const int32_t b0 = hrp[r], b1 = hrp[r + 1];
             if (b1 - b0 <= cut) continue;
             hl[t].x |= 1u << l;
@@ -1103,9 +1114,10 @@ static skf_status build_layout(skf_csr *A, int cut, int sort, cudaStream_t st) {
         k_sell_fill<<<blocks, 256, 0, st>>>(A->rowptr, A->colind, (const float *)A->values, n, A->nslices, cut,
                                             A->perm, A->sell_off, A->sell_w, (float *)A->sell_val, A->sell_col);
     count_launches(1);
+    const skf_status ds = build_diagonals(A, st);
     e = cudaStreamSynchronize(st);   // the host vectors above are released on return
     if (e != cudaSuccess) return cuda_fail(e, "SELL fill");
-    return build_diagonals(A, st);
+    return ds;
 }
 
 skf_status skf_create_csr(int64_t n, int64_t nnz, const int64_t *rowptr, const int32_t *colind, const void *values,

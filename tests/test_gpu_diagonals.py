@@ -44,10 +44,11 @@ def banded(n, offsets, keep=1.0, order="ascending", seed=5):
     return CSR(n, np.array(rowptr, dtype=np.int64), np.array(col, dtype=np.int32), np.array(val))
 
 
-# one ragged slice, several, a ragged last CTA, and a last slice of one row
+# one ragged slice, several, a ragged last CTA; from 16384 rows on the copy is
+# built: a last slice of one row
 # ("one" is not among them: on a diagonal of 3 +- 0.1 each FP64 column magnifies
 # the rounding of the one before 30-fold, whatever the kernel)
-@pytest.mark.parametrize("n", [29, 333, 5185])
+@pytest.mark.parametrize("n", [29, 5185, 16385])
 @pytest.mark.parametrize("name", sorted(set(OFFSETS) - {"one"}))
 @pytest.mark.parametrize("form,k", [("persistent", 2), ("persistent", 4), ("two_kernel", 2), ("two_kernel", 3),
                                     ("two_kernel", 6)])
@@ -61,12 +62,12 @@ def test_columns(skf, n, name, form, k):
 @pytest.mark.parametrize("order", ["ascending", "descending", "duplicate"])
 @pytest.mark.parametrize("form", ["persistent", "two_kernel"])
 def test_partly_filled_and_unordered_rows(skf, keep, order, form):
-    A = banded(1500, OFFSETS["five_uneven"], keep, order)
+    A = banded(17000, OFFSETS["five_uneven"], keep, order)
     mode = skf.ARNOLDI_PERSISTENT if form == "persistent" else skf.ARNOLDI_TWO_KERNEL
     check_columns(skf, A, gaussian_rhs(A.n, 3), 6, 2, 24, mode)
 
 
-@pytest.mark.parametrize("n", [333, 5185])
+@pytest.mark.parametrize("n", [333, 16385])
 @pytest.mark.parametrize("name", sorted(OFFSETS))
 @pytest.mark.parametrize("basis,form", [("f32", "persistent"), ("f32", "two_kernel"), ("bf16", "two_kernel")])
 def test_reduced_precision_sketches(skf, n, name, basis, form):
@@ -76,3 +77,14 @@ def test_reduced_precision_sketches(skf, n, name, basis, form):
         V, SV, SAV, H, info = arnoldi_lp(skf, A, gaussian_rhs(n, 3), m, 2, s, basis)
     assert info["m_eff"] == m
     check_sketches(A, V, SV, SAV, 2, s, m)
+
+
+# more slices per CTA than warps (several passes of the persistent kernel's loop)
+@pytest.mark.parametrize("name", ["six", "eight"])
+def test_many_slices_per_cta(skf, name):
+    A = banded(100_003, OFFSETS[name], 0.9)
+    b = gaussian_rhs(A.n, 3)
+    check_columns(skf, A, b, 5, 2, 24, skf.ARNOLDI_PERSISTENT)
+    V, SV, SAV, H, info = arnoldi_lp(skf, A, b, 5, 2, 24, "f32")
+    assert info["m_eff"] == 5
+    check_sketches(A, V, SV, SAV, 2, 24, 5)
