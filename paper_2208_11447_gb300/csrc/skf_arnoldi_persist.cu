@@ -65,7 +65,7 @@ struct PCtx {
     const void *sell_val;      // T values (T = double, or float for an FP32 basis)
     const int32_t *sell_col;
     DiagOp dg;                 // diagonal copy of the operator (dg.w = W, or 0: none)
-    float l2_frac;             // share of the operator's lines kept in L2 from step to step
+    float l2_frac;             // share of the operator's lines kept in L2 from step to step (not with y~ in global memory)
     SparseSign sp;
     const uint16_t *pattern;   // [n][zeta]
     const uint8_t *pattern8;   // [n][8] or nullptr
@@ -105,10 +105,15 @@ __device__ __forceinline__ int ld_volatile_i32(const int *p) {
 // whether it stays in L2 (129 MB) from one step to the next: `pol` keeps the
 // fraction l2_frac of its lines (evict_last) and streams the rest
 // (evict_first), so that an operator beyond the budget still finds that
-// fraction there instead of evicting itself.
+// fraction there instead of evicting itself.  A fraction lies in (0, 1]; an
+// operator of which nothing is kept (KEEP false) is streamed by a policy of its own.
+template <bool KEEP>
 __device__ __forceinline__ unsigned long long operator_policy(float frac) {
     unsigned long long p;
-    asm("createpolicy.fractional.L2::evict_last.L2::evict_first.b64 %0, %1;" : "=l"(p) : "f"(frac));
+    if constexpr (KEEP)
+        asm("createpolicy.fractional.L2::evict_last.L2::evict_first.b64 %0, %1;" : "=l"(p) : "f"(frac));
+    else
+        asm("createpolicy.fractional.L2::evict_first.b64 %0, 0f3F800000;" : "=l"(p));
     return p;
 }
 __device__ __forceinline__ double ld_op(const double *a, unsigned long long pol) {
@@ -413,13 +418,13 @@ __device__ __forceinline__ void scatter_row(const PCtx &c, int64_t r, uint2 pv, 
 // offsets of the window in win[], nw of them) and the magnitude key of
 // max|y~|.  Entries of one row are summed in their SELL (= CSR) order.
 constexpr int kSpmvWarps = kPNW - 1;   // the last warp serves the reductions
-template <int KW, int W, typename T>
+template <int KW, int W, bool KEEP, typename T>
 __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ wsrc, const T *win,
                                           const int (&soff)[KW], int nw, T *ys, const long long *meta_o,
                                           const int *meta_w, uint2 dmask, int nsl, int nr, T (&acc)[KW],
                                           unsigned &ykey) {
     const T *sell_val = (const T *)c.sell_val;
-    const unsigned long long pol = operator_policy(c.l2_frac);
+    const unsigned long long pol = operator_policy<KEEP>(c.l2_frac);
     const int lane = threadIdx.x & 31;
     int next_t = threadIdx.x >> 5;
     auto grab = [&]() {
@@ -833,8 +838,8 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
 #pragma unroll
             for (int a = 0; a < KW; ++a) soff[a] = a < nw ? ((i0 + a) % k) * R : 0;
             if (warp < kSpmvWarps)
-                spmv_rows<KW, W, T>(c, Vb + (size_t)j * c.ldv, win, soff, nw, ys, meta_o, meta_w, dmask, nsl, nr, acc,
-                                    ykey);
+                spmv_rows<KW, W, !YG, T>(c, Vb + (size_t)j * c.ldv, win, soff, nw, ys, meta_o, meta_w, dmask, nsl, nr,
+                                         acc, ykey);
         }
         if (flush_all && j >= 1) flush_w(j - 1, tid, kPT);
         __syncthreads();   // the bounds ea[] of the service warp
@@ -901,8 +906,8 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             for (int a = 0; a < KW; ++a) accb[a] = T(0);
             unsigned kb = 0;
             if (warp < kSpmvWarps)
-                spmv_rows<KW, W, T>(c, Vb + (size_t)jb * c.ldv, win, soff, 0, ys, meta_o, meta_w, dmask, nsl, nr, accb,
-                                    kb);
+                spmv_rows<KW, W, !YG, T>(c, Vb + (size_t)jb * c.ldv, win, soff, 0, ys, meta_o, meta_w, dmask, nsl, nr,
+                                         accb, kb);
             __syncthreads();
             const int ey = eys[jb & 3];
             const int shift_y = c.frac - (ey == kNoExp ? 0 : ey);
@@ -1189,15 +1194,9 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     c.sell_col = A->sell_col;
     // 8 diagonals of rows at most 7 wide: only the general FP64 form has 8 slots
     if (A->dia_w <= (f32 || yg ? 7 : 8)) c.dg = diag_of(A);
-    // L2 share of the operator, measured per step (keep none / this rule): all of
-    // it up to 90 MB (FP64 41.9 / 41.1 us at 84 MB, 21.6 / 20.2 at 22 MB; FP32
-    // 32.8 / 26.4 at 56 MB), beyond that 50 MB of it (FP32 47.8 / 45.2 at 97 MB;
-    // all of it 48.5).  With y~ in global memory L2 already holds that and the
-    // gathered vector, and a kept operator only displaces them (FP64 50.2 / 53.2
-    // at 106 MB, 49.3 / 52.9 at 84 MB): nothing is kept.
     const double opb = c.dg.w != 0 ? 32.0 * (double)A->nslices * (double)(vb * c.dg.w + 1)
                                    : (double)A->sell_entries * (double)(vb + 4);
-    c.l2_frac = yg ? 0.f : opb <= 90e6 ? 1.f : (float)(50e6 / opb);
+    c.l2_frac = l2_keep_fraction(opb);
     c.sp = make_sparse_sign(S);
     c.pattern = S->pattern;
     if (p8) {

@@ -282,6 +282,16 @@ __host__ __device__ __forceinline__ double scale_pow2(double x, int k) {
     return ldexp(x, k);
 }
 
+// Share of an operator of opb bytes that the persistent kernel keeps in L2 from
+// step to step, a fraction for createpolicy (valid range (0, 1]); measured per
+// step (keep none / this rule): all of it up to 90 MB (FP64 41.9 / 41.1 us at
+// 84 MB, 21.6 / 20.2 at 22 MB; FP32 32.8 / 26.4 at 56 MB), beyond that 50 MB of
+// it (FP32 47.8 / 45.2 at 97 MB; all of it 48.5).  With y~ in global memory L2
+// already holds that and the gathered vector, and a kept operator only displaces
+// them (FP64 50.2 / 53.2 at 106 MB, 49.3 / 52.9 at 84 MB): that form keeps
+// nothing, by a policy without a fraction.
+inline float l2_keep_fraction(double opb) { return opb <= 90e6 ? 1.f : (float)(50e6 / opb); }
+
 // 0 < xmax < inf (false for zero, negative, infinite and NaN xmax), with
 // integer instructions.
 __host__ __device__ __forceinline__ bool positive_finite(double xmax) {
