@@ -77,7 +77,7 @@ __device__ __forceinline__ void load_pattern(const uint16_t *pattern, int zeta, 
 // issue or by these atomics, not by memory.
 template <int OFF>
 __device__ __forceinline__ void red_shared(unsigned addr, int v) {
-    asm volatile("red.shared.add.s32 [%0+%2], %1;" ::"r"(addr), "r"(v), "n"(OFF));
+    asm volatile("red.shared.add.s32 [%0+%2], %1;" ::"r"(addr), "r"(v), "n"(OFF) : "memory");
 }
 template <int BLK, int LC, int Q = 0>
 __device__ __forceinline__ void scatter8(uint2 pv, unsigned base, int l0, int l1) {

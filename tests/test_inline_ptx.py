@@ -31,3 +31,18 @@ def test_policy_fractions_lie_in_range(tmp_path):
     assert res.returncode == 0, res.stderr
     run = subprocess.run([out], capture_output=True, text=True, timeout=120)
     assert run.returncode == 0, run.stdout + run.stderr
+
+
+
+def test_statements_that_access_memory_say_so():
+    """A statement that stores, or adds to memory, through an address the
+    compiler does not see carries the "memory" clobber: the sketch bins are
+    cleared and read by ordinary accesses on both sides."""
+    found, bare = 0, []
+    for name, text in sources():
+        for m in re.finditer(r"asm\s+volatile\s*\(((?:[^;\"]|\"[^\"]*\")*)\)\s*;", text):
+            if re.search(r"\"\s*(red|st|atom)\.", m.group(1)):
+                found += 1
+                if '"memory"' not in m.group(1):
+                    bare.append((name, m.group(1)))
+    assert found > 0 and not bare, bare
