@@ -79,8 +79,9 @@ struct PCtx {
     double *vscale, *SV, *SAV, *H;
     int *iscal;
     double *pB;                // [2][G]: partial ||b||^2, max|b|
-    unsigned long long *slot;  // [2 m + 1][kSlot]: exact sums of the window dots and max|y~| of step j at
-                               // 2 j, of ||w_j||^2, the Gram entries and max|w_j| at 2 j - 1 (see push_sums)
+    unsigned long long *slot;  // [3 m + 1][kSlot]: exact sums of the window dots and max|y~| of step j at
+                               // 2 j, of ||w_j||^2, the Gram entries and max|w_j| at 2 j - 1 (see push_sums),
+                               // of the dots below a tighter bound at 2 m + 1 + j
     int e_row;                 // |(A x)_r| < 2^e_row max|x|
     unsigned long long *accw;  // [m][2][s]: limb sums of S w_j
     unsigned long long *accy;  // [2][s]: limb sums of the directly sketched y~
@@ -254,11 +255,16 @@ __device__ __forceinline__ unsigned long long block_reduce_t0(double (&v)[NV], u
 // so after the barrier one 7-word load replaces the read and fixed-order sum
 // of G partials, and no FP64 addition (65 dependent cycles each on this part,
 // 16 more of the SM's FP64 pipe) is left on the path from the last row to the
-// coefficients.  The sums are exact to 2^-154 of the bound.  Measured per step
+// coefficients.  A partial is cut off 2^-154 below its bound and the sum 2^-132
+// below it (pull_sums carries the lowest chunk and drops the rest).  The bound of
+// the dots holds ||A||_inf, which one row can set far above the y~ of the others:
+// where it lies more than kMaxSlack bits above max|y~|, known after the barrier,
+// the dots are summed once more below that.  Measured per step
 // from the last row to the coefficients: 7.3 -> 5.9 us (100^3 grid, 152 CTAs),
 // 7.0 -> 4.2 us (10^4 rows; 10 -> 40 CTAs).
 constexpr int kCh = 7, kChBits = 22;         // chunks of a sum
 constexpr int kField = kCh * kChBits;        // bits below the bound
+constexpr int kMaxSlack = 60;                // bits by which the bound of the dots may lie above max|w_i| max|y~|
 constexpr int kSlot = 32;                    // words of a slot: kCh per sum (at most 4), [30] not finite, [31] max key
 
 // x as signed chunks of x / 2^(E - kField); false if x is not finite or not
@@ -609,7 +615,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
     __shared__ double fd[kMaxK], fg[KW][KW]; // MGS factors of the current step (phase A)
     __shared__ int ea[KW], eb[KW];           // exponent bounds of the per-thread sums of phases A and B
     __shared__ int sch[kSlot];               // this CTA's chunk sums (push_sums)
-    __shared__ int bar_ok;                   // the last grid barrier was passed
+    __shared__ int bar_ok;                   // the last grid barrier was passed (2: the dots are to be summed again)
     __shared__ int sbreak;                   // w_j is a happy breakdown
     unsigned nb = 0;                         // barriers passed
     const int nh = max(0, kSpmvWarps - nsl); // SpMV warps without a slice
@@ -843,8 +849,9 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
         }
         if (flush_all && j >= 1) flush_w(j - 1, tid, kPT);
         __syncthreads();   // the bounds ea[] of the service warp
-        {
-            unsigned long long *sl = c.slot + (size_t)(2 * j) * kSlot;
+        // grid sums of the dots and, by warp 0, the coefficients of the step; bar_ok
+        // becomes 2 where a first pass finds its bound too far above max|y~|
+        auto sum_dots = [&](unsigned long long *sl, bool first) {
             push_sums<KW, T>(acc, nw, ea, ykey, sch, sl);
             ++nb;
             if (warp == 0) {
@@ -887,9 +894,29 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
 #pragma unroll
                     for (int d = 1; d < KW; ++d)   // <w_{j+1}, w_{j+1-d}>
                         if (d <= nw) eb[d] = ew1 + ews[(j + 1 - d) & 3] + lg_rows;
+                    if (first && bar_ok && ey != kNoExp && ews[j & 3] + c.e_row - ey > kMaxSlack) bar_ok = 2;
                 }
             }
             __syncthreads();
+        };
+        sum_dots(c.slot + (size_t)(2 * j) * kSlot, true);
+        if (bar_ok != 1) {
+            if (bar_ok == 0) goto timeout;
+            // (rare) ||A||_inf says nothing about this y~: the dots once more, below
+            // max|y~|, from y~ and the window into the step's second slot
+            if (tid < nw) ea[tid] = ews[(i0 + tid) & 3] + eys[j & 3] + lg_rows;
+#pragma unroll
+            for (int a = 0; a < KW; ++a) acc[a] = T(0);
+            ykey = 0;
+            for (int lr = tid; lr < nr; lr += kPT) {
+                const T y = ys[lr];
+#pragma unroll
+                for (int a = 0; a < KW; ++a)
+                    if (a < nw) acc[a] = fma(win[((i0 + a) % k) * R + lr], y, acc[a]);
+                ykey = max(ykey, mag_key(y));
+            }
+            __syncthreads();
+            sum_dots(c.slot + (size_t)(2 * m + 1 + j) * kSlot, false);
             if (!bar_ok) goto timeout;
         }
 
@@ -1221,7 +1248,7 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
 
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t szP = sizeof(double) * 2 * (size_t)G;
-    const size_t szSlot = sizeof(unsigned long long) * (size_t)(2 * m + 1) * kSlot;
+    const size_t szSlot = sizeof(unsigned long long) * (size_t)(3 * m + 1) * kSlot;
     const size_t szAw = sizeof(unsigned long long) * (size_t)m * 2 * s;
     const size_t szAy = sizeof(unsigned long long) * 2 * (size_t)s;
     const size_t szSw = sizeof(double) * (size_t)s * m;
