@@ -522,15 +522,16 @@ static size_t dtype_size(skf_dtype d) { return d == SKF_F64 ? 8 : d == SKF_F32 ?
 
 static skf_status run_arnoldi(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, skf_dtype basis,
                               void *V, int64_t ldv, double *vscale, double *SV, double *SAV, double *H, int *iscal,
-                              skf_info *info, cudaStream_t cs, const StepHook *hook = nullptr, int vring = 0) {
+                              skf_info *info, cudaStream_t cs, const StepHook *hook = nullptr, int vring = 0,
+                              int lanes = 1) {
     if (basis == SKF_F64)
-        return arnoldi_run(A, S, b, m, k, (double *)V, ldv, vscale, SV, SAV, H, iscal, info, cs, hook, vring);
+        return arnoldi_run(A, S, b, m, k, (double *)V, ldv, vscale, SV, SAV, H, iscal, info, cs, hook, vring, lanes);
     if (basis == SKF_F32) {
         // the persistent form where it applies (as for FP64: no per-step hooks,
         // one-pass storage), else the two-kernel form
         if (step_mode() != 1 && hook == nullptr && vring == 0) {
             const skf_status ps =
-                arnoldi_run_persistent_f32(A, S, b, m, k, (float *)V, ldv, vscale, SV, SAV, H, iscal, info, cs);
+                arnoldi_run_persistent_f32(A, S, b, m, k, (float *)V, ldv, vscale, SV, SAV, H, iscal, info, cs, lanes);
             if (ps != SKF_ERR_NOT_SUPPORTED) return ps;
             if (step_mode() == 2) return fail(SKF_ERR_NOT_SUPPORTED, "persistent Arnoldi form does not apply here");
         }
@@ -636,9 +637,11 @@ static skf_status solve_check(skf_method method, const skf_csr *A, const skf_ske
 }
 
 // Enqueue one validated solve on `cs`: stream-ordered workspace, the
-// Arnoldi process, the tail, release of the workspace.
+// Arnoldi process, the tail, release of the workspace.  lanes: of the batch it
+// belongs to.
 static skf_status solve_enqueue(skf_method method, const skf_csr *A, const skf_sketch *S, const void *b,
-                                const skf_params &p, void *x, skf_info *info, const RuleDev &rule, cudaStream_t cs) {
+                                const skf_params &p, void *x, skf_info *info, const RuleDev &rule, cudaStream_t cs,
+                                int lanes = 1) {
     const int m = p.m;
     const int64_t n = A->n;
     const int s = S->s;
@@ -702,7 +705,7 @@ static skf_status solve_enqueue(skf_method method, const skf_csr *A, const skf_s
         iscal2 = (int *)(ws + off); off += al(sizeof(int) * 4);
     }
     st = run_arnoldi(A, S, (const double *)b, m, p.k, bt, V, ldv, vscale, SV, SAV, H, iscal, info, cs,
-                     stopping ? &hook : nullptr, vring);
+                     stopping ? &hook : nullptr, vring, lanes);
     if (st == SKF_OK && sc.err != SKF_OK) st = sc.err;
     if (st == SKF_OK)
         st = tail_run(method, s, m, n, V, bt, ldv, vscale, SV, SAV, iscal, rule, p.tol, two ? nullptr : (double *)x,
@@ -1569,7 +1572,7 @@ skf_status skf_solve_batched(int32_t nprob, const skf_problem *probs, int32_t la
     for (int i : order) {
         if (st != SKF_OK) break;
         const skf_problem &q = probs[i];
-        st = solve_enqueue(q.method, q.A, q.S, q.b, *q.p, q.x, q.info, *rules[i], pool->s[lane_of[i]]);
+        st = solve_enqueue(q.method, q.A, q.S, q.b, *q.p, q.x, q.info, *rules[i], pool->s[lane_of[i]], L);
         if (st != SKF_OK) err = "problem " + std::to_string(i) + ": " + skf_last_error();
     }
     for (int l = 0; l < L; ++l) {

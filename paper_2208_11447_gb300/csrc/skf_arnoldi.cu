@@ -872,11 +872,11 @@ void launch_steps_k(const ArnCtx &c, int G, int Gs, size_t smem, const SrhtDev *
 // Host driver: launches init, m x (spmv, update), finish on `st`.
 skf_status arnoldi_run(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, double *V, int64_t ldv,
                        double *vscale, double *SV, double *SAV, double *H, int *iscal, skf_info *info,
-                       cudaStream_t st, const StepHook *hook, int vring) {
+                       cudaStream_t st, const StepHook *hook, int vring, int lanes) {
     // the persistent single-launch form where it applies (no per-step host
     // hooks, one-pass storage, sparse-sign S, k <= 4, rows fit in shared memory)
     if (step_mode() != 1 && hook == nullptr && vring == 0) {
-        const skf_status ps = arnoldi_run_persistent(A, S, b, m, k, V, ldv, vscale, SV, SAV, H, iscal, info, st);
+        const skf_status ps = arnoldi_run_persistent(A, S, b, m, k, V, ldv, vscale, SV, SAV, H, iscal, info, st, lanes);
         if (ps != SKF_ERR_NOT_SUPPORTED) return ps;
         if (step_mode() == 2) return fail(SKF_ERR_NOT_SUPPORTED, "persistent Arnoldi form does not apply here");
     }

@@ -51,9 +51,22 @@ namespace {
 
 constexpr int kPT = 512;                      // threads per CTA
 constexpr int kPNW = kPT / 32;                // warps per CTA
-// rows per CTA below which CTAs are left out: 10^4 rows 12.4 / 9.6 / 9.6 us
-// per step at 512 / 256 / 128 rows, 25600 rows 13.7 / 10.6 / 10.9 us
-constexpr int kPersistMinRows = 256;
+// Rows per CTA below which CTAs are left out.  Alone, 10^4 rows take 12.4 / 9.6 /
+// 9.6 us per step at 512 / 256 / 128 rows, 25600 rows 13.7 / 10.6 / 10.9 us.  The
+// solves of a batch on three or more lanes share the card: they take the first
+// level at which those of all lanes leave a quarter of it (at two CTAs per SM) to
+// each other's tails, else the last.  16 solves with m = 40, ms per batch with
+// 1024 rows and one CTA per SM / 256 rows and one CTA per SM / the levels: 1e4 rows
+// on 8 lanes 2.56 / 3.02 / 2.16, 25600 on 4 lanes 4.43 / 6.90 / 4.00 and on 8 3.13 /
+// 6.97 / 2.73, 4e4 on 8 4.39 / 7.46 / 3.69, four operators of 1e4 to 1e5 rows on 8
+// 4.90 / 7.00 / 3.91.
+constexpr int kPersistMinRows[kPersistLevels] = {256, 384, 768};
+// Rows per CTA up to which a partition takes the short form of the kernel: two
+// CTAs per SM (64 registers; a warp has at most three slices, so nothing is
+// loaded ahead), and sums that do not depend on the partition (a summand is a
+// lane's share of one or two slices, see persist_group), so that a solve gives the
+// same bits alone and in a batch.
+constexpr int kShortRows = 1024;
 constexpr int kFlushAll = 64;                 // slices per CTA up to which all warps add up the sketch bins
 constexpr long long kBarrierBudget = 1ll << 31;   // SM cycles (about one second)
 
@@ -65,6 +78,7 @@ struct PCtx {
     const void *sell_val;      // T values (T = double, or float for an FP32 basis)
     const int32_t *sell_col;
     DiagOp dg;                 // diagonal copy of the operator (dg.w = W, or 0: none)
+    int group;                 // (short form) slices per summand of the grid sums, 1 or 2 (persist_group)
     float l2_frac;             // share of the operator's lines kept in L2 from step to step (not with y~ in global memory)
     SparseSign sp;
     const uint16_t *pattern;   // [n][zeta]
@@ -78,7 +92,7 @@ struct PCtx {
     int64_t ldv;
     double *vscale, *SV, *SAV, *H;
     int *iscal;
-    double *pB;                // [2][G]: partial ||b||^2, max|b|
+    double *pB;                // [2][G]: partial ||b||^2, max|b| (short form: [2][slices])
     unsigned long long *slot;  // [3 m + 1][kSlot]: exact sums of the window dots and max|y~| of step j at
                                // 2 j, of ||w_j||^2, the Gram entries and max|w_j| at 2 j - 1 (see push_sums),
                                // of the dots below a tighter bound at 2 m + 1 + j
@@ -247,29 +261,33 @@ __device__ __forceinline__ unsigned long long block_reduce_t0(double (&v)[NV], u
 }
 
 // Grid-wide sums without floating-point additions.  The per-thread partials of
-// a phase (window dots; ||w||^2 and Gram entries) are cut into kCh chunks of
-// 22 bits of a 154-bit field below an exponent bound that every CTA knows, and
+// a phase (window dots; ||w||^2 and Gram entries) are cut into kCh chunks of 22
+// bits (short form: 21) of a field below an exponent bound that every CTA knows, and
 // the chunks are added as integers: a warp reduction per chunk, a shared
 // atomic per warp, one 64-bit global atomic per CTA and chunk, issued just
 // before the CTA's barrier arrival.  Integer sums do not depend on the order,
 // so after the barrier one 7-word load replaces the read and fixed-order sum
 // of G partials, and no FP64 addition (65 dependent cycles each on this part,
 // 16 more of the SM's FP64 pipe) is left on the path from the last row to the
-// coefficients.  A partial is cut off 2^-154 below its bound and the sum 2^-132
-// below it (pull_sums carries the lowest chunk and drops the rest).  The bound of
+// coefficients.  A partial is cut off 2^-154 (2^-147) below its bound and the sum
+// 2^-132 (2^-126) below it (pull_sums carries the lowest chunk and drops the rest).  The bound of
 // the dots holds ||A||_inf, which one row can set far above the y~ of the others:
 // where it lies more than kMaxSlack bits above max|y~|, known after the barrier,
 // the dots are summed once more below that.  Measured per step
 // from the last row to the coefficients: 7.3 -> 5.9 us (100^3 grid, 152 CTAs),
 // 7.0 -> 4.2 us (10^4 rows; 10 -> 40 CTAs).
-constexpr int kCh = 7, kChBits = 22;         // chunks of a sum
-constexpr int kField = kCh * kChBits;        // bits below the bound
-constexpr int kMaxSlack = 60;                // bits by which the bound of the dots may lie above max|w_i| max|y~|
+// The short form has up to kShortRows summands per CTA: 21-bit chunks there, so
+// that a CTA's sum stays below 2^31.
+constexpr int kCh = 7;                                   // chunks of a sum
+constexpr int chunk_bits(bool sh) { return sh ? 21 : 22; }
+constexpr int kMaxSlack = 54;                // bits by which the bound of the dots may lie above max|w_i| max|y~|
 constexpr int kSlot = 32;                    // words of a slot: kCh per sum (at most 4), [30] not finite, [31] max key
 
-// x as signed chunks of x / 2^(E - kField); false if x is not finite or not
-// below 2^E in magnitude.
+// x as signed chunks of CB bits of x / 2^(E - kCh CB); false if x is not finite
+// or not below 2^E in magnitude.
+template <int CB>
 __device__ __forceinline__ bool chunks_of(double x, int E, int (&ch)[kCh]) {
+    constexpr int kField = kCh * CB;
     const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
     const int be = (int)((bits >> 52) & 0x7FFull);
     const unsigned long long mant = be ? ((bits & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) : 0ull;
@@ -278,16 +296,18 @@ __device__ __forceinline__ bool chunks_of(double x, int E, int (&ch)[kCh]) {
     const bool neg = (bits >> 63) != 0ull;
 #pragma unroll
     for (int i = 0; i < kCh; ++i) {
-        const int sh = kChBits * i - p;
+        const int sh = CB * i - p;
         unsigned long long v;
         asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(mant), "r"(max(sh, 0)));   // shifts of 64 and more give 0
         asm("shl.b64 %0, %1, %2;" : "=l"(v) : "l"(v), "r"(max(-sh, 0)));
-        const int d = (int)((unsigned)v & ((1u << kChBits) - 1u));
+        const int d = (int)((unsigned)v & ((1u << CB) - 1u));
         ch[i] = ok ? (neg ? -d : d) : 0;
     }
     return ok;
 }
+template <int CB>
 __device__ __forceinline__ bool chunks_of(float x, int E, int (&ch)[kCh]) {
+    constexpr int kField = kCh * CB;
     const unsigned bits = __float_as_uint(x);
     const int be = (int)((bits >> 23) & 0xFFu);
     const unsigned mant = be ? ((bits & 0x7FFFFFu) | 0x800000u) : 0u;
@@ -296,11 +316,11 @@ __device__ __forceinline__ bool chunks_of(float x, int E, int (&ch)[kCh]) {
     const bool neg = (bits >> 31) != 0u;
 #pragma unroll
     for (int i = 0; i < kCh; ++i) {
-        const int sh = kChBits * i - p;
+        const int sh = CB * i - p;
         unsigned v;
         asm("shr.u32 %0, %1, %2;" : "=r"(v) : "r"(mant), "r"(max(sh, 0)));
         asm("shl.b32 %0, %1, %2;" : "=r"(v) : "r"(v), "r"(max(-sh, 0)));
-        const int d = (int)(v & ((1u << kChBits) - 1u));
+        const int d = (int)(v & ((1u << CB) - 1u));
         ch[i] = ok ? (neg ? -d : d) : 0;
     }
     return ok;
@@ -324,32 +344,31 @@ __device__ __forceinline__ int exponent_above(double x) {
     return (int)(mag_key(x) >> 20) - 1022;
 }
 
-// Adds the first nv of the per-thread values v[] (|v[i]| < 2^E[i]) and the
-// maximum of the keys to this CTA's share of `slot`: warp reductions, shared
-// atomics, then one global atomic per chunk from warp 0, whose lane 0 may
-// arrive at the barrier after a __syncwarp().  sch: kSlot ints, zero on entry
-// and left zero.
-template <int KW, typename T>
-__device__ __forceinline__ void push_sums(const T (&v)[KW], int nv, const int *E, unsigned key, int *sch,
-                                          unsigned long long *slot) {
+// One value of every thread of the warp (|v| < 2^E) into value a's chunk sums:
+// lane a kCh + i holds the warp's sum of chunk i in `mine`, `bad` a value that
+// is not finite.
+template <int CB, typename T>
+__device__ __forceinline__ void add_chunks(T v, int E, int a, int &mine, bool &bad) {
     const int lane = threadIdx.x & 31;
-    int mine = 0;
-    bool bad = false;
+    int ch[kCh];
+    bad |= !chunks_of<CB>(v, E, ch);
 #pragma unroll
-    for (int a = 0; a < KW; ++a) {
-        if (a < nv) {
-            int ch[kCh];
-            bad |= !chunks_of(v[a], E[a], ch);
-#pragma unroll
-            for (int i = 0; i < kCh; ++i) {
-                const int t = __reduce_add_sync(0xffffffffu, ch[i]);   // |t| < 2^27
-                if (lane == a * kCh + i) mine = t;
-            }
-        }
+    for (int i = 0; i < kCh; ++i) {
+        const int t = __reduce_add_sync(0xffffffffu, ch[i]);   // |t| < 2^(CB + 5)
+        if (lane == a * kCh + i) mine += t;
     }
+}
+
+// Adds the warps' chunk sums of nv values and the maximum of the keys to this
+// CTA's share of `slot`: shared atomics (at most 2^(31 - CB) summands per CTA),
+// then one global atomic per chunk from warp 0, whose lane 0 may arrive at the
+// barrier after a __syncwarp().  sch: kSlot ints, zero on entry and left zero.
+__device__ __forceinline__ void flush_sums(int mine, bool bad, int nv, unsigned key, int *sch,
+                                           unsigned long long *slot) {
+    const int lane = threadIdx.x & 31;
     key = __reduce_max_sync(0xffffffffu, key);
     bad = __any_sync(0xffffffffu, bad);
-    if (lane < nv * kCh) atomicAdd(sch + lane, mine);                   // 512 (2^22 - 1) < 2^31
+    if (lane < nv * kCh) atomicAdd(sch + lane, mine);
     if (lane == 30 && bad) sch[30] = 1;
     if (lane == 31) atomicMax((unsigned *)sch + 31, key);
     __syncthreads();
@@ -362,11 +381,24 @@ __device__ __forceinline__ void push_sums(const T (&v)[KW], int nv, const int *E
     }
 }
 
+// The first nv of the per-thread values v[] (|v[i]| < 2^E[i]).
+template <int CB, int KW, typename T>
+__device__ __forceinline__ void push_sums(const T (&v)[KW], int nv, const int *E, unsigned key, int *sch,
+                                          unsigned long long *slot) {
+    int mine = 0;
+    bool bad = false;
+#pragma unroll
+    for (int a = 0; a < KW; ++a)
+        if (a < nv) add_chunks<CB>(v[a], E[a], a, mine, bad);
+    flush_sums(mine, bad, nv, key, sch, slot);
+}
+
 // The sums of a slot (after the barrier): lane i < nv returns value i (carries
 // from the lowest chunk up, then the digits as three integers and two FMAs;
 // NaN when a partial was not finite), every lane the slot's maximum key.  One
 // load per chunk and lane: a single coalesced load of the slot and shuffles
 // took 3.4 instead of 1.8 us with 152 CTAs reading it (1.9 / 1.3 with 40).
+template <int CB>
 __device__ __forceinline__ double pull_sums(const unsigned long long *slot, int nv, const int *E, unsigned &key) {
     const int lane = threadIdx.x & 31;
     const unsigned long long *p = slot + (lane < nv ? lane : 0) * kCh;
@@ -376,17 +408,17 @@ __device__ __forceinline__ double pull_sums(const unsigned long long *slot, int 
     key = (unsigned)__ldcg(slot + 31);
     const bool bad = __ldcg(slot + 30) != 0ull;
     if (lane >= nv) return 0.0;
-    constexpr long long mask = (1ll << kChBits) - 1;
+    constexpr long long mask = (1ll << CB) - 1;
 #pragma unroll
     for (int q = 0; q + 1 < kCh; ++q) {
-        t[q + 1] += t[q] >> kChBits;
+        t[q + 1] += t[q] >> CB;
         t[q] &= mask;
     }
-    const long long hi = t[6] * (1ll << kChBits) + t[5];
-    const long long mid = (t[4] << kChBits) | t[3], lo = (t[2] << kChBits) | t[1];
-    constexpr double two44 = 17592186044416.0;
-    const double r = fma(fma((double)hi, two44, (double)mid), two44, (double)lo);
-    return bad ? __longlong_as_double(0x7FF8000000000000ll) : scale_pow2(r, E[lane] - kField + kChBits);
+    const long long hi = t[6] * (1ll << CB) + t[5];
+    const long long mid = (t[4] << CB) | t[3], lo = (t[2] << CB) | t[1];
+    constexpr double two = (double)(1ull << (2 * CB));
+    const double r = fma(fma((double)hi, two, (double)mid), two, (double)lo);
+    return bad ? __longlong_as_double(0x7FF8000000000000ll) : scale_pow2(r, E[lane] - (kCh - 1) * CB);
 }
 
 // Fixed-point limbs of one value into the shared bins of the sparse-sign
@@ -424,7 +456,7 @@ __device__ __forceinline__ void scatter_row(const PCtx &c, int64_t r, uint2 pv, 
 // offsets of the window in win[], nw of them) and the magnitude key of
 // max|y~|.  Entries of one row are summed in their SELL (= CSR) order.
 constexpr int kSpmvWarps = kPNW - 1;   // the last warp serves the reductions
-template <int KW, int W, bool KEEP, typename T>
+template <int KW, int W, bool KEEP, bool SHORT, typename T>
 __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ wsrc, const T *win,
                                           const int (&soff)[KW], int nw, T *ys, const long long *meta_o,
                                           const int *meta_w, uint2 dmask, int nsl, int nr, T (&acc)[KW],
@@ -438,6 +470,49 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
         next_t += kSpmvWarps;
         return t;
     };
+    if constexpr (SHORT) {   // y~ alone: the dots follow from shared memory
+        for (int t = next_t; t < nsl; t += kSpmvWarps) {
+            T y = T(0);
+            if (W > 0 && c.dg.w != 0) {
+                constexpr int WD = W > 0 ? W : 1;
+                const int64_t r0 = (int64_t)blockIdx.x * c.R + 32 * t + lane;
+                const unsigned m = t == next_t ? dmask.x : t == next_t + kSpmvWarps ? dmask.y
+                                                                                   : (unsigned)__ldg(c.dg.mask + r0);
+                const T *dv = (const T *)c.dg.val + (r0 - lane) * W + lane;
+                const T *wr = wsrc + r0;
+                T av[WD], xv[WD];
+#pragma unroll
+                for (int d = 0; d < W; ++d) {
+                    av[d] = ld_op(dv + 32 * d, pol);
+                    xv[d] = (m >> d) & 1u ? __ldcg(wr + c.dg.off[d]) : T(0);
+                }
+#pragma unroll
+                for (int d = 0; d < W; ++d) y = fma(av[d], xv[d], y);
+            } else {
+                const int wt = meta_w[t];
+                const T *pv = sell_val + meta_o[t] + lane;
+                const int32_t *pc = c.sell_col + meta_o[t] + lane;
+                if constexpr (W > 0) {
+                    T av[W], xv[W];
+                    int cv[W];
+#pragma unroll
+                    for (int p = 0; p < W; ++p) cv[p] = p < wt ? ld_op(pc + 32 * p, pol) : 0;
+#pragma unroll
+                    for (int p = 0; p < W; ++p) av[p] = p < wt ? ld_op(pv + 32 * p, pol) : T(0);
+#pragma unroll
+                    for (int p = 0; p < W; ++p) xv[p] = p < wt ? __ldcg(wsrc + cv[p]) : T(0);
+#pragma unroll
+                    for (int p = 0; p < W; ++p)
+                        if (p < wt) y = fma(av[p], xv[p], y);
+                } else {
+                    for (int p = 0; p < wt; ++p)
+                        y = fma(ld_op(pv + 32 * p, pol), __ldcg(wsrc + ld_op(pc + 32 * p, pol)), y);
+                }
+            }
+            if (t * 32 + lane < nr) ys[t * 32 + lane] = y;
+        }
+        return;
+    }
     if (W > 0 && c.dg.w != 0) {
         // diagonal copy: values and gathers of slice tn and the masks of slice
         // tnn in flight while slice t is computed (a row past nr is present in no
@@ -577,9 +652,10 @@ __device__ __forceinline__ void spmv_rows(const PCtx &c, const T *__restrict__ w
 // orthogonalisation and accumulation, the update applying the FP32 values of
 // sigma_j and of the MGS coefficients (H and S A v_j are those of the relation
 // with the applied values), everything else FP64.
-template <int KW, int W, int ZCAP, bool YG, typename T>
-__global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
+template <int KW, int W, int ZCAP, bool YG, bool SHORT, typename T>
+__global__ void __launch_bounds__(kPT, SHORT ? 2 : 1) k_arnoldi_persist(PCtx c) {
     constexpr bool F32 = sizeof(T) == 4;
+    constexpr int CB = chunk_bits(SHORT);
     extern __shared__ __align__(16) unsigned char psm[];
     constexpr int kRed = kPT + 4 + kPNW;             // block_reduce_t0<1>
     constexpr int kSvc = kPNW - 1;                   // the service warp
@@ -619,7 +695,11 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
     __shared__ int sbreak;                   // w_j is a happy breakdown
     unsigned nb = 0;                         // barriers passed
     const int nh = max(0, kSpmvWarps - nsl); // SpMV warps without a slice
-    const int lg_rows = 32 - __clz(R / 256); // log2 of a bound of the rows one thread sums
+    // (short form) slices per group less one, and this thread's row at its turn q:
+    // warp w takes the groups w, w + kPNW, ..., slice by slice
+    const int gl = SHORT ? c.group - 1 : 0;
+    auto row_of = [&](int q) { return ((((warp + kPNW * (q >> gl)) << gl) | (q & gl)) << 5) | lane; };
+    const int lg_rows = SHORT ? gl : 32 - __clz(R / 256); // log2 of a bound of the products in one summand
 
     // Column i of S V and column i-1 of S A V from the integer sums of S w_i
     // (rows is = g + G t of S): S w_i, S v_i = sigma_i S w_i and, by the
@@ -721,7 +801,31 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
     }
     if (tid == 0) sbreak = 0;
     if (tid < kSlot) sch[tid] = 0;
-    {
+    if constexpr (SHORT) {
+        // sums of b^2 by slice, which the partition does not change
+        const int64_t ns = (c.n + 31) >> 5;
+        for (int t = warp; t < nsl; t += kPNW) {
+            const int lr = t * 32 + lane;
+            double v = 0.0, mx = 0.0;
+            if (lr < nr) {
+                const T xt = (T)c.b[r0 + lr];
+                const double x = (double)xt;
+                Vb[r0 + lr] = xt;
+                win[lr] = xt;    // slot 0
+                v = x * x;
+                mx = key_to_abs(abs_key(x));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                v += __shfl_xor_sync(0xffffffffu, v, o);
+                mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            }
+            if (lane == 0) {
+                c.pB[r0 / 32 + t] = v;
+                c.pB[ns + r0 / 32 + t] = mx;
+            }
+        }
+    } else {
         double nrm[1] = {0.0};
         unsigned long long key = 0;
         for (int lr = tid; lr < nr; lr += kPT) {
@@ -739,7 +843,32 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
         }
     }
     if (!grid_barrier(c.bar, c.flag, ++nb, c.budget)) goto timeout;
-    if (warp < 2) {
+    if constexpr (SHORT) {
+        // by 128 threads, whatever the grid
+        const int ns = (int)((c.n + 31) >> 5);
+        if (warp < 4) {
+            double v = 0.0, mx = 0.0;
+#pragma unroll 4
+            for (int t = tid; t < ns; t += 128) {
+                v += __ldcg(c.pB + t);
+                mx = fmax(mx, __ldcg(c.pB + ns + t));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                v += __shfl_xor_sync(0xffffffffu, v, o);
+                mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            }
+            if (lane == 0) {
+                red[warp] = v;
+                red[4 + warp] = mx;
+            }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            sb[0] = ((red[0] + red[1]) + red[2]) + red[3];
+            sb[1] = fmax(fmax(red[4], red[5]), fmax(red[6], red[7]));
+        }
+    } else if (warp < 2) {
         const double v = reduce_slot(c.pB + (size_t)warp * G, G, warp == 1);
         if (lane == 0) sb[warp] = v;
     }
@@ -780,7 +909,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
         if (warp == kSvc && j >= 1) {
             // lane 0: ||w_j||^2, lane d: <w_j, w_{j-d}>
             unsigned wk;
-            const double tot = pull_sums(c.slot + (size_t)(2 * j - 1) * kSlot, 1 + ngj, eb, wk);
+            const double tot = pull_sums<CB>(c.slot + (size_t)(2 * j - 1) * kSlot, 1 + ngj, eb, wk);
             double gr[KW];
 #pragma unroll
             for (int d = 1; d < KW; ++d) gr[d] = __shfl_sync(0xffffffffu, tot, d);
@@ -839,20 +968,41 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             if (j >= 2)
                 for (int t = ht; g + G * t < s; t += nt) finalize_col(j - 2, t);
         }
-        {
-            int soff[KW];   // window slot offsets, oldest first
+        int soff[KW];   // window slot offsets, oldest first
 #pragma unroll
-            for (int a = 0; a < KW; ++a) soff[a] = a < nw ? ((i0 + a) % k) * R : 0;
-            if (warp < kSpmvWarps)
-                spmv_rows<KW, W, !YG, T>(c, Vb + (size_t)j * c.ldv, win, soff, nw, ys, meta_o, meta_w, dmask, nsl, nr,
-                                         acc, ykey);
-        }
+        for (int a = 0; a < KW; ++a) soff[a] = a < nw ? ((i0 + a) % k) * R : 0;
+        if (warp < kSpmvWarps)
+            spmv_rows<KW, W, !YG, SHORT, T>(c, Vb + (size_t)j * c.ldv, win, soff, nw, ys, meta_o, meta_w, dmask, nsl,
+                                            nr, acc, ykey);
         if (flush_all && j >= 1) flush_w(j - 1, tid, kPT);
         __syncthreads();   // the bounds ea[] of the service warp
         // grid sums of the dots and, by warp 0, the coefficients of the step; bar_ok
         // becomes 2 where a first pass finds its bound too far above max|y~|
         auto sum_dots = [&](unsigned long long *sl, bool first) {
-            push_sums<KW, T>(acc, nw, ea, ykey, sch, sl);
+            if constexpr (SHORT) {
+                int mine = 0;
+                bool bad = false;
+                unsigned key = 0;
+                for (int q = 0; row_of(q) - lane < nr; ++q) {   // a summand per lane and turn
+                    T v[KW];
+#pragma unroll
+                    for (int a = 0; a < KW; ++a) v[a] = T(0);
+                    for (int u = 0; u <= gl; ++u, q += u <= gl) {
+                        const int lr = row_of(q);
+                        const T y = lr < nr ? ys[lr] : T(0);
+#pragma unroll
+                        for (int a = 0; a < KW; ++a)
+                            if (a < nw && lr < nr) v[a] = fma(win[soff[a] + lr], y, v[a]);
+                        key = max(key, mag_key(y));
+                    }
+#pragma unroll
+                    for (int a = 0; a < KW; ++a)
+                        if (a < nw) add_chunks<CB>(v[a], ea[a], a, mine, bad);
+                }
+                flush_sums(mine, bad, nw, key, sch, sl);
+            } else {
+                push_sums<CB, KW, T>(acc, nw, ea, ykey, sch, sl);
+            }
             ++nb;
             if (warp == 0) {
                 __syncwarp();
@@ -865,7 +1015,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
                 // w_{i0+a}; MGS in the window, ascending, from the dots and the Gram
                 // matrix: h_i = <v_i, y> - sum_{i' < i} h_i' <v_i, v_i'>
                 unsigned yk;
-                double dot = pull_sums(sl, nw, ea, yk);
+                double dot = pull_sums<CB>(sl, nw, ea, yk);
                 if (lane < nw) dot *= fd[lane];
                 double h[KW];
 #pragma unroll
@@ -905,15 +1055,17 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             // (rare) ||A||_inf says nothing about this y~: the dots once more, below
             // max|y~|, from y~ and the window into the step's second slot
             if (tid < nw) ea[tid] = ews[(i0 + tid) & 3] + eys[j & 3] + lg_rows;
+            if constexpr (!SHORT) {
 #pragma unroll
-            for (int a = 0; a < KW; ++a) acc[a] = T(0);
-            ykey = 0;
-            for (int lr = tid; lr < nr; lr += kPT) {
-                const T y = ys[lr];
+                for (int a = 0; a < KW; ++a) acc[a] = T(0);
+                ykey = 0;
+                for (int lr = tid; lr < nr; lr += kPT) {
+                    const T y = ys[lr];
 #pragma unroll
-                for (int a = 0; a < KW; ++a)
-                    if (a < nw) acc[a] = fma(win[((i0 + a) % k) * R + lr], y, acc[a]);
-                ykey = max(ykey, mag_key(y));
+                    for (int a = 0; a < KW; ++a)
+                        if (a < nw) acc[a] = fma(win[soff[a] + lr], y, acc[a]);
+                    ykey = max(ykey, mag_key(y));
+                }
             }
             __syncthreads();
             sum_dots(c.slot + (size_t)(2 * m + 1 + j) * kSlot, false);
@@ -933,7 +1085,7 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             for (int a = 0; a < KW; ++a) accb[a] = T(0);
             unsigned kb = 0;
             if (warp < kSpmvWarps)
-                spmv_rows<KW, W, !YG, T>(c, Vb + (size_t)jb * c.ldv, win, soff, 0, ys, meta_o, meta_w, dmask, nsl, nr,
+                spmv_rows<KW, W, !YG, SHORT, T>(c, Vb + (size_t)jb * c.ldv, win, soff, 0, ys, meta_o, meta_w, dmask, nsl, nr,
                                          accb, kb);
             __syncthreads();
             const int ey = eys[jb & 3];
@@ -987,37 +1139,54 @@ __global__ void __launch_bounds__(kPT, 1) k_arnoldi_persist(PCtx c) {
             for (int a = 0; a < KW; ++a) part[a] = T(0);
             unsigned nkey = 0;
             uint2 pv_next = make_uint2(0u, 0u);
-            if (p8 && tid < nr) pv_next = __ldg((const uint2 *)(c.pattern8 + (r0 + tid) * 8));
-            for (int lr = tid; lr < nr; lr += kPT) {
+            int mine = 0;      // (short form: chunk sums)
+            bool bad = false;
+            // rows of this thread; in the short form whole groups, lanes past nr without a row
+            int lr = SHORT ? row_of(0) : tid;
+            if (p8 && lr < nr) pv_next = __ldg((const uint2 *)(c.pattern8 + (r0 + lr) * 8));
+            for (int q = 0; SHORT ? lr - lane < nr || (q & gl) != 0 : lr < nr; ++q) {
                 const int64_t r = r0 + lr;
+                const int lrn = SHORT ? row_of(q + 1) : lr + kPT;
                 const uint2 pv = pv_next;
-                if (p8 && lr + kPT < nr) pv_next = __ldg((const uint2 *)(c.pattern8 + (r + kPT) * 8));
-                const T y = ys[lr];
-                T wv[KW];
+                if (p8 && lrn < nr) pv_next = __ldg((const uint2 *)(c.pattern8 + (r0 + lrn) * 8));
+                if (!SHORT || lr < nr) {
+                    const T y = ys[lr];
+                    T wv[KW];
 #pragma unroll
-                for (int b2 = 0; b2 < KW; ++b2) wv[b2] = b2 < nw ? win[soffr[b2] + lr] : T(0);
-                if (!last) {
-                    T w = sj * y;
+                    for (int b2 = 0; b2 < KW; ++b2) wv[b2] = b2 < nw ? win[soffr[b2] + lr] : T(0);
+                    if (!last) {
+                        T w = sj * y;
 #pragma unroll
-                    for (int b2 = KW - 1; b2 >= 0; --b2)
-                        if (b2 < nw) w = fma(-cf[b2], wv[b2], w);   // oldest first
-                    wn[r] = w;
-                    win[snew + lr] = w;
-                    part[0] = fma(w, w, part[0]);
-                    nkey = max(nkey, mag_key(w));
+                        for (int b2 = KW - 1; b2 >= 0; --b2)
+                            if (b2 < nw) w = fma(-cf[b2], wv[b2], w);   // oldest first
+                        wn[r] = w;
+                        win[snew + lr] = w;
+                        nkey = max(nkey, mag_key(w));
+                        part[0] = fma(w, w, part[0]);
 #pragma unroll
-                    for (int d = 1; d < KW; ++d)
-                        if (d <= ng) part[d] = fma(w, wv[d - 1], part[d]);
+                        for (int d = 1; d < KW; ++d)
+                            if (d <= ng) part[d] = fma(w, wv[d - 1], part[d]);
+                    }
+                    const long long vw = ew == kNoExp ? 0 : fixed_point(wv[0], shift_w);
+                    scatter_row<ZCAP>(c, r, pv, p8, bw0, bw1, (int)(vw & lmask), (int)(vw >> c.L));
+                    if (last) {
+                        const long long vy = ey == kNoExp ? 0 : fixed_point(y, shift_y);
+                        scatter_row<ZCAP>(c, r, pv, p8, by0, by1, (int)(vy & lmask), (int)(vy >> c.L));
+                    }
                 }
-                const long long vw = ew == kNoExp ? 0 : fixed_point(wv[0], shift_w);
-                scatter_row<ZCAP>(c, r, pv, p8, bw0, bw1, (int)(vw & lmask), (int)(vw >> c.L));
-                if (last) {
-                    const long long vy = ey == kNoExp ? 0 : fixed_point(y, shift_y);
-                    scatter_row<ZCAP>(c, r, pv, p8, by0, by1, (int)(vy & lmask), (int)(vy >> c.L));
+                if (SHORT && !last && (q & gl) == gl) {   // the group's summands
+#pragma unroll
+                    for (int d = 0; d < KW; ++d) {
+                        if (d <= ng) add_chunks<CB>(part[d], eb[d], d, mine, bad);
+                        part[d] = T(0);
+                    }
                 }
+                lr = lrn;
             }
             if (!last) {
-                push_sums<KW, T>(part, 1 + ng, eb, nkey, sch, c.slot + (size_t)(2 * j + 1) * kSlot);
+                unsigned long long *sl = c.slot + (size_t)(2 * j + 1) * kSlot;
+                if constexpr (SHORT) flush_sums(mine, bad, 1 + ng, nkey, sch, sl);
+                else push_sums<CB, KW, T>(part, 1 + ng, eb, nkey, sch, sl);
             } else {
                 __syncthreads();
                 flush_w(j, tid, kPT);
@@ -1086,6 +1255,14 @@ __global__ void k_persist_info(const double *__restrict__ vscale, const int *__r
     info->eps_est = __longlong_as_double((long long)*epsmax);
 }
 
+// The short form (kShortRows) and its slices per summand, by the size alone,
+// whatever the partition of a call: with one slice per summand the cutting into
+// chunks, about 100 instructions per warp and value, would come twice per phase
+// beyond 512 rows per CTA (N = 1e5, m = 40: 858 us, 801 with two slices and the
+// window offsets taken out of the loop; alone on the card at one CTA per SM, 781).
+bool persist_short(int64_t n) { return n <= (int64_t)kShortRows * num_sms(); }
+int persist_group(int64_t n) { return n <= (int64_t)kPT * num_sms() ? 1 : 2; }
+
 // A barrier that can never complete (it waits for one CTA more than the
 // grid has), with the given budget: the self-test of the bounded wait.
 __global__ void __launch_bounds__(32) k_barrier_selftest(unsigned *bar, int *flag, long long budget, int *status) {
@@ -1096,7 +1273,9 @@ __global__ void __launch_bounds__(32) k_barrier_selftest(unsigned *bar, int *fla
 
 template <int KW, int W, int ZCAP, bool YG, typename T>
 cudaError_t launch_persist(const PCtx &c, int G, size_t smem, cudaStream_t st) {
-    auto kern = k_arnoldi_persist<KW, W, ZCAP, YG, T>;
+    auto kern = k_arnoldi_persist<KW, W, ZCAP, YG, false, T>;
+    if constexpr (!YG)
+        if (persist_short(c.n)) kern = k_arnoldi_persist<KW, W, ZCAP, false, true, T>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -1153,16 +1332,30 @@ size_t persist_smem(int R, int k, int nbin, bool yg, size_t vb = sizeof(double))
 
 }  // namespace
 
-// Persistent partition: G = min(SMs, ceil(n / kPersistMinRows)) CTAs of R rows
-// (whole slices).  The sketch tables record the bin-load maximum of this
-// partition.
-void persist_partition(int64_t n, int *G, int64_t *rows) {
-    int64_t g = (n + kPersistMinRows - 1) / kPersistMinRows;
+// Persistent partition of a level: G = min(SMs, ceil(n / kPersistMinRows)) CTAs
+// of R rows (whole slices).  The sketch tables record the bin-load maximum over
+// the levels.
+void persist_partition(int64_t n, int level, int *G, int64_t *rows) {
+    const int64_t mr = kPersistMinRows[level];
+    int64_t g = (n + mr - 1) / mr;
     if (g > num_sms()) g = num_sms();
     if (g < 1) g = 1;
-    const int64_t R = ((n + g - 1) / g + 31) / 32 * 32;
+    const int64_t u = persist_short(n) ? 32 * persist_group(n) : 32;   // whole groups
+    const int64_t R = ((n + g - 1) / g + u - 1) / u * u;
     *rows = R;
     *G = (int)((n + R - 1) / R);
+}
+
+// The level of a solve on one of `lanes` lanes (beyond kShortRows all levels are one).
+static int persist_level(int64_t n, int lanes) {
+    if (lanes <= 2) return 0;   // (two of any size fit side by side)
+    for (int l = 0; l + 1 < kPersistLevels; ++l) {
+        int G;
+        int64_t rows;
+        persist_partition(n, l, &G, &rows);
+        if (2ll * lanes * G <= 3ll * num_sms()) return l;
+    }
+    return kPersistLevels - 1;
 }
 
 static int g_step_mode = 0;   // 0 auto, 1 two-kernel path only, 2 persistent path required
@@ -1174,7 +1367,7 @@ int step_mode() { return g_step_mode; }
 // N up to about 2e6).
 static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, void *V,
                                  int64_t ldv, double *vscale, double *SV, double *SAV, double *H, int *iscal,
-                                 skf_info *info, cudaStream_t st, bool f32) {
+                                 skf_info *info, cudaStream_t st, bool f32, int lanes) {
     if (S->kind != SKF_SKETCH_SPARSE_SIGN || S->binmax_persist == nullptr || k > 4 ||
         A->vdtype != (f32 ? SKF_F32 : SKF_F64) || A->nlong > 0 ||
         A->perm != nullptr)   // a row split or sorted slices take the two-kernel form
@@ -1183,7 +1376,7 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     const size_t vb = f32 ? sizeof(float) : sizeof(double);
     int G;
     int64_t R64;
-    persist_partition(A->n, &G, &R64);
+    persist_partition(A->n, persist_level(A->n, lanes), &G, &R64);
     if (G > kMaxG) return SKF_ERR_NOT_SUPPORTED;
     const int R = (int)R64;
     const int KW = k <= 2 ? 2 : 4;
@@ -1215,6 +1408,7 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     PCtx c{};
     c.n = A->n;
     c.R = R;
+    c.group = persist_group(A->n);
     c.sell_off = A->sell_off;
     c.sell_w = A->sell_w;
     c.sell_val = A->sell_val;
@@ -1247,7 +1441,7 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
     c.budget = kBarrierBudget;
 
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t szP = sizeof(double) * 2 * (size_t)G;
+    const size_t szP = sizeof(double) * 2 * (size_t)(persist_short(A->n) ? (A->n + 31) / 32 : G);
     const size_t szSlot = sizeof(unsigned long long) * (size_t)(3 * m + 1) * kSlot;
     const size_t szAw = sizeof(unsigned long long) * (size_t)m * 2 * s;
     const size_t szAy = sizeof(unsigned long long) * 2 * (size_t)s;
@@ -1299,14 +1493,14 @@ static skf_status run_persistent(const skf_csr *A, const skf_sketch *S, const do
 
 skf_status arnoldi_run_persistent(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, double *V,
                                   int64_t ldv, double *vscale, double *SV, double *SAV, double *H, int *iscal,
-                                  skf_info *info, cudaStream_t st) {
-    return run_persistent(A, S, b, m, k, V, ldv, vscale, SV, SAV, H, iscal, info, st, false);
+                                  skf_info *info, cudaStream_t st, int lanes) {
+    return run_persistent(A, S, b, m, k, V, ldv, vscale, SV, SAV, H, iscal, info, st, false, lanes);
 }
 
 skf_status arnoldi_run_persistent_f32(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, float *V,
                                       int64_t ldv, double *vscale, double *SV, double *SAV, double *H, int *iscal,
-                                      skf_info *info, cudaStream_t st) {
-    return run_persistent(A, S, b, m, k, V, ldv, vscale, SV, SAV, H, iscal, info, st, true);
+                                      skf_info *info, cudaStream_t st, int lanes) {
+    return run_persistent(A, S, b, m, k, V, ldv, vscale, SV, SAV, H, iscal, info, st, true, lanes);
 }
 
 // Self-test of the bounded barrier wait: a grid of `ctas` co-resident CTAs

@@ -189,7 +189,7 @@ struct skf_sketch {
     uint16_t *pattern = nullptr;
     int *binmax = nullptr;            // device: most nonzeros one CTA row range puts in one row of S
     int *binmax_chunk = nullptr;      // device: the same for the chunk-interleaved partition
-    int *binmax_persist = nullptr;    // device: the same for the persistent partition (persist_partition)
+    int *binmax_persist = nullptr;    // device: the same for the persistent partitions (persist_partition)
     int binmax_persist_host = 0;      // host copy of *binmax_persist
     // Compact pattern when every stripe has at most 128 rows and zeta <= 8:
     // byte [c * 8 + q] = (row of nonzero q within stripe q) + p8_block * sign,
@@ -484,7 +484,8 @@ void chunk_partition(int64_t n, int *G);
 
 // Row partition of the persistent FP64 Arnoldi kernel: G <= SMs CTAs of
 // `rows` consecutive rows each (whole SELL slices), every CTA non-empty.
-void persist_partition(int64_t n, int *G, int64_t *rows);
+constexpr int kPersistLevels = 3;
+void persist_partition(int64_t n, int level, int *G, int64_t *rows);
 
 // Fixed-point sketch accumulation.  A value x is rounded to the integer
 // v = x 2^(P - E) (E: exponent bound of the vector, |v| < 2^P) and split into
@@ -559,11 +560,11 @@ inline void call_col_hook(const StepHook *h, int j, cudaStream_t st) {
 // fit it (sketch kind, k > 4, shared memory, cooperative launch).
 skf_status arnoldi_run_persistent(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, double *V,
                                   int64_t ldv, double *vscale, double *SV, double *SAV, double *H, int *iscal,
-                                  skf_info *info, cudaStream_t st);
+                                  skf_info *info, cudaStream_t st, int lanes);
 // the persistent form with an FP32 basis (FP32 values, k <= 2, slices at most 7 wide)
 skf_status arnoldi_run_persistent_f32(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, float *V,
                                       int64_t ldv, double *vscale, double *SV, double *SAV, double *H, int *iscal,
-                                      skf_info *info, cudaStream_t st);
+                                      skf_info *info, cudaStream_t st, int lanes);
 // Which FP64 step form arnoldi_run uses: 0 automatic (persistent where it
 // fits), 1 the two-kernel form only, 2 the persistent form or
 // SKF_ERR_NOT_SUPPORTED.
@@ -582,7 +583,7 @@ skf_status barrier_selftest(int ctas, long long budget, int *status_out, cudaStr
 
 skf_status arnoldi_run(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, double *V, int64_t ldv,
                        double *vscale, double *SV, double *SAV, double *H, int *iscal, skf_info *info,
-                       cudaStream_t st, const StepHook *hook = nullptr, int vring = 0);
+                       cudaStream_t st, const StepHook *hook = nullptr, int vring = 0, int lanes = 1);
 // Reduced-precision variants: FP32 matrix values, basis stored in FP32 or
 // BF16 (V of that type), FP32 SpMV and orthogonalisation, FP64 sketches.
 skf_status arnoldi_run_f32(const skf_csr *A, const skf_sketch *S, const double *b, int m, int k, float *V,

@@ -342,11 +342,17 @@ skf_status build_sparse_sign_tables(skf_sketch *S, cudaStream_t st) {
     int Gc;
     chunk_partition(S->n, &Gc);
     k_bin_max<<<Gc, 256, smem, st>>>(sp, S->n, kChunkRows, S->pattern, S->binmax_chunk);
-    int Gp;
-    int64_t rows_p;
-    persist_partition(S->n, &Gp, &rows_p);
-    k_bin_max<<<Gp, 256, smem, st>>>(sp, S->n, rows_p, S->pattern, S->binmax_persist);
-    count_launches(4);
+    int64_t last_rows = 0;   // the persistent partitions, where they differ
+    for (int level = 0; level < kPersistLevels; ++level) {
+        int Gp;
+        int64_t rows_p;
+        persist_partition(S->n, level, &Gp, &rows_p);
+        if (rows_p == last_rows) continue;
+        last_rows = rows_p;
+        k_bin_max<<<Gp, 256, smem, st>>>(sp, S->n, rows_p, S->pattern, S->binmax_persist);
+        count_launches(1);
+    }
+    count_launches(3);
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "sketch table build");
     int hmax[3] = {0, 0, 0};
