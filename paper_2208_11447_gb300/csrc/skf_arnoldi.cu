@@ -23,8 +23,9 @@
 // update's own rounding (about one unit roundoff of ||A v_j||), as in the
 // persistent form.  Only the last S y~ (and with the stopping criterion those of
 // the steps before a checkpoint, so that a checkpoint sees what a run of that
-// length sees) is sketched directly; at a happy breakdown the noise vector w_{m_eff} is sketched once more to close the last
-// relation.  One sketched vector per step instead of two, the update's shared
+// length sees) is sketched directly, and at a happy breakdown, where w_{m_eff}
+// may be noise or not finite, that of the step before it.
+// One sketched vector per step instead of two, the update's shared
 // atomics (16 per row and vector) and the SRDCT's transforms halved:
 // N = 4.0e6, zeta = 8: update 77 -> 66 us; SRDCT at N = 3.6e5: one transform
 // per step instead of two.
@@ -114,7 +115,8 @@ __device__ __forceinline__ double sketch_row(const long long *part, int G, int s
 // S w_jw from the partials of its step (an SRDCT has written it) for this
 // CTA's slice of the rows of S; then S A v_{jw-1} by the relation (see above)
 // unless it is sketched directly; with `store` (jw < m_eff) S v_jw and, where
-// y~_jw is sketched directly, S A v_jw from its partials.
+// y~_jw is sketched directly, S A v_jw from its partials.  Without it (a happy
+// breakdown at jw) the step sketched y~_{jw-1} in the place of w_jw.
 __device__ __forceinline__ void finalize_column(const ArnCtx &c, int jw, bool store) {
     const bool rel = jw >= 1 && !y_direct(c, jw - 1), ydir = store && !c.direct && y_direct(c, jw);
     const int s = c.sp.s;
@@ -132,8 +134,8 @@ __device__ __forceinline__ void finalize_column(const ArnCtx &c, int jw, bool st
             if (!c.direct) c.Sw[(size_t)jw * s + i] = sw;
             if (store) c.SV[i + (size_t)jw * s] = c.vscale[jw] * sw;
             if (rel) {
-                double v = sw;
-                for (int b = nw - 1; b >= 0; --b) v = fma(cf[b], c.Sw[(size_t)(jw - 1 - b) * s + i], v);
+                double v = store ? sw : c.vscale[jw - 1] * sw;
+                for (int b = store ? nw - 1 : -1; b >= 0; --b) v = fma(cf[b], c.Sw[(size_t)(jw - 1 - b) * s + i], v);
                 c.SAV[i + (size_t)(jw - 1) * s] = v;
             }
             if (ydir) c.SAV[i + (size_t)jw * s] = c.vscale[jw] * sy;
@@ -519,7 +521,9 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // stopped at this step (set by its SpMV launch) or earlier; at a happy
-    // breakdown at this step only w_j is sketched
+    // breakdown at this step y~_{j-1}, still in Y, is sketched in the place of w_j
+    // (which need not be finite: the products of the step may have overflowed); a
+    // dense sketch, applied to the slot of w_j after this launch, finds it there
     const bool stop_here = c.iscal[0] == 1 && c.iscal[3] == j && j >= 1;
     if (c.iscal[0] && c.iscal[3] <= j && (!stop_here || c.identity)) return;
     const int G = gridDim.x;
@@ -572,7 +576,7 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     const int L = c.sparse ? limb_bits(*c.binmax) : 0;
     const int frac = sketch_fraction_bits_from_limb(L);
     const long long lmask = (1ll << L) - 1;
-    const int ew = positive_finite(wmax) ? bound_exponent(wmax) : kNoExp;
+    const int ew = stop_here ? c.eys[j - 1] : positive_finite(wmax) ? bound_exponent(wmax) : kNoExp;
     if (blockIdx.x == 0 && threadIdx.x == 0) c.ews[j] = ew;
     const int shift_w = frac - (ew == kNoExp ? 0 : ew);
     const int shift_y = frac - (ey == kNoExp ? 0 : ey);
@@ -586,6 +590,11 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     unsigned long long nkey = 0;
     const int64_t r0 = (int64_t)blockIdx.x * c.rows_per_cta;
     const int64_t r1 = min(c.n, r0 + c.rows_per_cta);
+    if (stop_here && !c.sparse) {
+        double *wj = c.V + vcol(c, j);
+        for (int64_t r = r0 + threadIdx.x; r < r1; r += kUpdThreads) wj[r] = c.Y[r];
+        return;
+    }
     double *wn = c.V + vcol(c, j + 1);
     // window offsets newest first: woffr[b] locates w_{j-b}
     int64_t woffr[KW];
@@ -630,7 +639,7 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
             if (xr < rn) {
                 const int64_t r = r0 + xr;
                 const double y = cur.y[u];
-                const double wjr = cur.w[u][0];
+                const double wjr = stop_here ? y : cur.w[u][0];
                 if (do_update) {
                     double w = sigma * y;
 #pragma unroll
@@ -744,7 +753,7 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
 
 // After the loop: the pending columns.  Ran to the end: S v_{m-1}, S A v_{m-2}
 // by the relation and the sketched S A v_{m-1}.  Happy breakdown at step me:
-// S w_me (not a basis column) gives S A v_{me-1}.
+// S y~_{me-1}, sketched at that step, gives S A v_{me-1}.
 __global__ void __launch_bounds__(kThreads) k_arnoldi_finish(ArnCtx c) {
     const int me = c.iscal[1];
     if (me == 0 || c.identity || c.iscal[0] == 2) return;   // (2: stopped by the criterion, columns < me are final)
