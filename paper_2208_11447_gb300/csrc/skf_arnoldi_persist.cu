@@ -290,9 +290,9 @@ __device__ __forceinline__ bool chunks_of(double x, int E, int (&ch)[kCh]) {
     constexpr int kField = kCh * CB;
     const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
     const int be = (int)((bits >> 52) & 0x7FFull);
-    const unsigned long long mant = be ? ((bits & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) : 0ull;
-    const int p = be - 1075 - (E - kField);   // position of the mantissa's lowest bit in the field
-    const bool ok = be != 0x7FF && (be == 0 || p <= kField - 53);
+    const unsigned long long frac = bits & 0xFFFFFFFFFFFFFull, mant = be ? frac | 0x10000000000000ull : frac;
+    const int p = max(be, 1) - 1075 - (E - kField);   // position of the mantissa's lowest bit in the field
+    const bool ok = be != 0x7FF && (mant == 0ull || p + 64 - __clzll((long long)mant) <= kField);
     const bool neg = (bits >> 63) != 0ull;
 #pragma unroll
     for (int i = 0; i < kCh; ++i) {
@@ -310,9 +310,9 @@ __device__ __forceinline__ bool chunks_of(float x, int E, int (&ch)[kCh]) {
     constexpr int kField = kCh * CB;
     const unsigned bits = __float_as_uint(x);
     const int be = (int)((bits >> 23) & 0xFFu);
-    const unsigned mant = be ? ((bits & 0x7FFFFFu) | 0x800000u) : 0u;
-    const int p = be - 150 - (E - kField);
-    const bool ok = be != 0xFF && (be == 0 || p <= kField - 24);
+    const unsigned frac = bits & 0x7FFFFFu, mant = be ? frac | 0x800000u : frac;
+    const int p = max(be, 1) - 150 - (E - kField);
+    const bool ok = be != 0xFF && (mant == 0u || p + 32 - __clz((int)mant) <= kField);
     const bool neg = (bits >> 31) != 0u;
 #pragma unroll
     for (int i = 0; i < kCh; ++i) {

@@ -55,3 +55,13 @@ def test_solve_of_an_overflowing_process(skf, form):
         torch.cuda.synchronize()
         assert skf.read_info(info)["status"] == 0
         assert 0.0 < float(x.norm()) * 1e134 < float(b.norm())
+
+
+# ||w_1||^2 about 1e-308 and below: its summands are subnormal; the second step's
+# norm is gone and ends the process in both forms
+@pytest.mark.parametrize("form", ["persistent", "two_kernel"])
+@pytest.mark.parametrize("scale", [1e-158, 1e-160])
+def test_subnormal_norms_count(skf, form, scale):
+    A, S, V, SAV, info = columns(skf, form, scale)
+    assert info["breakdown"] == 1 and info["m_eff"] == 2
+    assert rel(SAV[0], S @ (csr_to_scipy(A) @ V[0])) < 1e-11
