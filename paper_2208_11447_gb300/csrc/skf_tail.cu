@@ -241,7 +241,7 @@ size_t qr_smem_bytes(int s) {
 
 __global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, double *pub, int *flag) {
     extern __shared__ double qsm[];
-    __shared__ double qsc[2];       // u_0 and 1 / D of the current reflector
+    __shared__ double qsc[3];       // u_0, 1 / D of the current reflector; sign(x0) ||x|| where 1 / D leaves the range
     __shared__ double qf[kQrOwn];   // factors f of the columns being updated
     const int me = c.iscal[1];
     const int ncols = c.rel ? me + 1 : 2 * me;
@@ -329,7 +329,9 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, double *pu
         // x(jj+1:)], H = I - u u^T / D, D = ||x|| (||x|| + |x0|), and the factor of
         // a column y is f = (u_0 y(jj) + x^T y) / D (a quotient with the LAPACK
         // scaling of u and its two more products were half of the 1.3 us this
-        // takes on the chain).  By warp 0 only: a warp instruction occupies the
+        // takes on the chain).  Where D or 1 / D leaves the range of a double
+        // (||x|| below 1e-154 or above 1e154), f = (y(jj) + x^T y / u_0) / (sign(x0) ||x||),
+        // the same quotient in two steps.  By warp 0 only: a warp instruction occupies the
         // FP64 pipe for 16 cycles whatever its active lanes, so scalar FP64 work
         // repeated by every warp costs eight times the pipe time.
         if (warp0) {
@@ -337,7 +339,7 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, double *pu
             const bool upd = lane < n1 && kf < nq;
             const double xy = upd ? qr_total(tot, nv1, 1 + lane) : 0.0;
             const double yj = upd ? cols[(size_t)(kf + lane) * s + jj] : 0.0;
-            double beta = x0, u0 = 0.0, di = 0.0;
+            double beta = x0, u0 = 0.0, di = 0.0, nxe = 0.0;
             if (sig > 0.0 || x0 == 0.0) {
                 const double q2 = fma(x0, x0, sig);
                 if (q2 > 0.0) {
@@ -346,14 +348,19 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, double *pu
                     di = 1.0 / fma(x0, nx, q2);
                     u0 = x0 + nx;
                     beta = -nx;
+                    if ((unsigned)(__double2hiint(di) - 1) >= 0x7FEFFFFFu) {   // 0, inf (or NaN)
+                        di = 1.0;
+                        nxe = nx;
+                    }
                 }
             }
             if (lane == 0) {
                 qsc[0] = u0;
                 qsc[1] = di;
+                qsc[2] = nxe;
                 if (writer) c.Rdiag[jj] = beta;
             }
-            if (upd) qf[lane] = fma(u0, yj, xy) * di;
+            if (upd) qf[lane] = __double2hiint(nxe) ? (yj + xy / u0) / nxe : fma(u0, yj, xy) * di;
         }
         __syncthreads();
         if (kf >= nq) continue;
@@ -392,8 +399,11 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_persist(TailCtx c, double *pu
                 }
                 __syncthreads();   // (qf[0] has been read by every thread)
                 qr_block_sums(loc, n2, sm, tot);
-                if (warp0 && lane < n2)
-                    qf[lane] = fma(u0, cols[(size_t)(kf + 1 + lane) * s + jj], qr_total(tot, n2, lane)) * di;
+                if (warp0 && lane < n2) {
+                    const double yj = cols[(size_t)(kf + 1 + lane) * s + jj], xy = qr_total(tot, n2, lane);
+                    const double nxe = qsc[2];
+                    qf[lane] = __double2hiint(nxe) ? (yj + xy / u0) / nxe : fma(u0, yj, xy) * di;
+                }
                 __syncthreads();
                 if (di != 0.0) {
 #pragma unroll
