@@ -953,10 +953,12 @@ static void free_layout(skf_csr *A) {
 // Small operators keep the slices: they live in L2 and a step is latency (10^4 rows:
 // 9.9 us per step with the slices, 10.0 with the copy; 25600 rows: 9.8 and 9.6), while
 // the copy's launches and allocation add 0.3 ms to the upload.
+// FP64 operators beyond the persistent form's sizes keep them too: the two-kernel
+// FP64 product does not read the copy (159^3: 229 MB, 256^3: 956 MB).
 constexpr int64_t kDiagMinRows = 16384;
 static skf_status build_diagonals(skf_csr *A, cudaStream_t st) {
     const size_t esz = A->vdtype == SKF_F64 ? 8 : 4;
-    if (A->n < kDiagMinRows) return SKF_OK;
+    if (A->n < kDiagMinRows || (A->vdtype == SKF_F64 && A->n > persist_max_rows_f64())) return SKF_OK;
     if (A->perm != nullptr || A->nlong > 0 || A->max_width > 8 || A->nnz == 0) return SKF_OK;
     int *tab = nullptr, h[9];
     if (dalloc((void **)&tab, sizeof(h), st) != SKF_OK) return SKF_OK;

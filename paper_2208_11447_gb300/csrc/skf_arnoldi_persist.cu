@@ -1346,6 +1346,18 @@ void persist_partition(int64_t n, int level, int *G, int64_t *rows) {
     *G = (int)((n + R - 1) / R);
 }
 
+int64_t persist_max_rows_f64() {
+    int dev = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    int R = 32;
+    while (persist_smem(R + 32, 2, 16 * 64, true) + 4096 <= (size_t)optin) R += 32;
+    return (int64_t)R * num_sms();
+}
+
 // The level of a solve on one of `lanes` lanes (beyond kShortRows all levels are one).
 static int persist_level(int64_t n, int lanes) {
     if (lanes <= 2) return 0;   // (two of any size fit side by side)

@@ -486,6 +486,8 @@ void chunk_partition(int64_t n, int *G);
 // `rows` consecutive rows each (whole SELL slices), every CTA non-empty.
 constexpr int kPersistLevels = 3;
 void persist_partition(int64_t n, int level, int *G, int64_t *rows);
+// rows up to which the persistent form holds an FP64 basis (k = 2, a sketch of few rows)
+int64_t persist_max_rows_f64();
 
 // Fixed-point sketch accumulation.  A value x is rounded to the integer
 // v = x 2^(P - E) (E: exponent bound of the vector, |v| < 2^P) and split into
