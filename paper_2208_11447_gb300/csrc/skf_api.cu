@@ -765,15 +765,9 @@ static skf_status lane_pool(LanePool **out) {
     return SKF_OK;
 }
 
-// Estimated device seconds of one problem: m steps, each the larger of its
-// streamed bytes at HBM speed and a launch-latency floor, plus a tail that
-// grows with m (Householder columns and quadrature nodes).
 static double solve_cost(const skf_problem &q) {
-    const double vb = (double)dtype_size(q.p->basis_dtype);
-    const double ab = (double)dtype_size(q.A->vdtype) + 4.0;
-    const double bytes = (double)q.A->nnz * ab + 3.0 * (double)q.A->n * vb;
-    const double step = std::max(bytes / 6.0e12, 12.0e-6);
-    return q.p->m * (step + 40.0e-6);
+    return solve_seconds(q.p->m, (double)q.A->n, (double)q.A->nnz, (int)dtype_size(q.A->vdtype),
+                         (int)dtype_size(q.p->basis_dtype));
 }
 
 // Longest-processing-time-first: problems by decreasing cost, each onto the

@@ -484,6 +484,18 @@ void chunk_partition(int64_t n, int *G);
 
 // Row partition of the persistent FP64 Arnoldi kernel: G <= SMs CTAs of
 // `rows` consecutive rows each (whole SELL slices), every CTA non-empty.
+// Estimated device seconds of a solve, by which a batch is dealt out to its lanes:
+// m steps, each the larger of its streamed bytes and of the latency of its grid
+// barriers, plus a tail that grows with m (reflectors and node solves).  Measured
+// per step: FP64 9.6 us at 1e4 rows, 34.5 at 1e6 (107 MB: 3.1 TB/s), 150 at 4.0e6
+// (2.9); FP32 23.6 at 1e6 (2.9), 230 at 1.7e7 (5.0), BF16 53 at 3.4e6 (3.9); tail 6.3
+// to 6.7 us per column (m = 40 and 240), in the full form of a BF16 basis about 40.
+inline double solve_seconds(int m, double n, double nnz, int value_bytes, int basis_bytes) {
+    const double bytes = nnz * (value_bytes + 4.0) + 3.0 * n * basis_bytes;
+    const double step = bytes / (basis_bytes == 8 ? 3.1e12 : 4.0e12);
+    return m * ((step > 9.6e-6 ? step : 9.6e-6) + (basis_bytes == 2 ? 40e-6 : 6.5e-6));
+}
+
 constexpr int kPersistLevels = 3;
 void persist_partition(int64_t n, int level, int *G, int64_t *rows);
 // rows up to which the persistent form holds an FP64 basis (k = 2, a sketch of few rows)
