@@ -20,7 +20,6 @@ def test_short_columns(skf, N, noalloc):
     for scale in (1e30, 1.0):
         X = g.standard_normal((N, 3)) * scale
         X[:, 1] = 0.0
-        X[0, 2] = -1e3 * scale
         got = apply(S, torch.as_tensor(X, device="cuda")).cpu().numpy()
         want = O @ X
         assert not got[:, 1].any()
