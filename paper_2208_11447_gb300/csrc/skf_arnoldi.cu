@@ -840,16 +840,16 @@ void launch_steps(const ArnCtx &c, int G, int Gs, size_t smem, const SrhtDev *sd
         // the process stopped before step j: a breakdown at step j still needs S w_j)
         double *wj = c.V + (size_t)(c.vring ? j % c.vring : j) * c.ldv;
         if (dd) {   // S w_j, and SAV[:, j] = sigma_j S y_j
-            for (int q = 0; q < (ydir ? 2 : 1); ++q) {
-                SrdctCols cols{};
-                cols.ncols = 1;
-                cols.x[0] = q == 0 ? wj : c.Y;
-                cols.out[0] = q == 0 ? c.Sw + (size_t)j * c.sp.s : c.SAV + (size_t)j * c.sp.s;
-                cols.colscale = q == 0 ? nullptr : c.stepsc + 4 * (size_t)j;
-                cols.iscal = c.iscal;
-                cols.step = q == 0 ? j - 1 : j;
-                srdct_launch(*dd, cols, st);
-            }
+            SrdctCols cols{};
+            cols.ncols = ydir ? 2 : 1;
+            cols.x[0] = wj;
+            cols.out[0] = c.Sw + (size_t)j * c.sp.s;
+            cols.x[1] = c.Y;   // (at a breakdown at step j a column past the last)
+            cols.out[1] = c.SAV + (size_t)j * c.sp.s;
+            cols.colscale[1] = c.stepsc + 4 * (size_t)j;
+            cols.iscal = c.iscal;
+            cols.step = j - 1;
+            srdct_launch(*dd, cols, st);
         }
         if (sd) {   // S w_j, and S y_j (exponents written by the update kernel)
             SrhtCols cols{};

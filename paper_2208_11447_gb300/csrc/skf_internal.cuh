@@ -710,7 +710,7 @@ struct SrdctDev {
 struct SrdctCols {
     const void *x[2];    // F64 columns, or F32 with f32 = 1 (widened exactly)
     double *out[2];
-    const double *colscale;
+    const double *colscale[2];   // factor of the column (device), or nullptr
     int ncols;
     const int *iscal;
     int step;

@@ -71,8 +71,8 @@ __global__ void __launch_bounds__(kSrdctThreads) k_srdct(SrdctDev d, SrdctCols c
     block_sum<2>(acc, red);
     if (threadIdx.x == 0) {
         const double sk = sqrt((k == 0 ? 1.0 : 2.0) / (double)d.s);
-        const double cscale = cols.colscale ? *cols.colscale : 1.0;
-        for (int q = 0; q < cols.ncols; ++q) cols.out[q][i] = acc[q] * sk * cscale;
+        for (int q = 0; q < cols.ncols; ++q)
+            cols.out[q][i] = acc[q] * sk * (cols.colscale[q] ? *cols.colscale[q] : 1.0);
     }
 }
 
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dct_gather(SrdctDev d, SrdctCol
     const int q = blockIdx.y;
     const int64_t L = d.fft_len;
     const double2 *Z = Zall + (size_t)q * L;
-    const double cscale = cols.colscale ? *cols.colscale : 1.0;
+    const double cscale = cols.colscale[q] ? *cols.colscale[q] : 1.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.s; i += gridDim.x * blockDim.x) {
         const int64_t k = d.P[i];
         double2 V;
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(kDotThreads) k_dct_dots(SrdctDev d, SrdctCols 
     double2 V = make_double2(v[0], v[1]);
     if (packed) V = unpack_v(V, make_double2(v[2], v[3]), d.tw[k]);
     const double2 t = d.twist[i];
-    cols.out[q][i] = fma(t.x, V.x, -t.y * V.y) * (cols.colscale ? *cols.colscale : 1.0);
+    cols.out[q][i] = fma(t.x, V.x, -t.y * V.y) * (cols.colscale[q] ? *cols.colscale[q] : 1.0);
 }
 
 RootTable root_table(int R) {
@@ -458,7 +458,10 @@ skf_status build_srdct_tables(skf_sketch *S) {
         for (int i = 0; i < nrad; ++i) S->rad[i] = rad[i];
         // pruned form: P1 = the most leading radices whose product stays within
         // kGroupMax, where summing the rest directly (8 s P2 FMAs with the pair of
-        // outputs) costs less than the passes it replaces (about 2.5 L log2 P2 FMAs)
+        // outputs) costs less than the passes it replaces (about 2.5 L log2 P2 FMAs).
+        // 20 Arnoldi steps, full passes / pruned: N = 4e4 1.83 / 1.15 ms at s = 240,
+        // 1.89 / 1.30 at s = 800 (1200: full); N = 3.6e5 2.54 / 1.56 and 2.55 / 1.79;
+        // N = 1e6 4.38 / 2.88 and 4.41 / 3.14, at s = 2000 4.45 / 3.56
         int64_t p1 = 1;
         for (int i = 0; i < nrad && p1 * rad[i] <= kGroupMax; ++i) p1 *= rad[i];
         const int64_t p2 = len / p1;

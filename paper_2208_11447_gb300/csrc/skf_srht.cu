@@ -251,8 +251,8 @@ void dense_sketch_f32(const skf_sketch *S, const DenseCols &cols, void *work, cu
         for (int q = 0; q < cols.ncols; ++q) {
             sc.x[q] = cols.x[q];
             sc.out[q] = cols.out[q];
+            sc.colscale[q] = cols.colscale;
         }
-        sc.colscale = cols.colscale;
         sc.iscal = cols.iscal;
         sc.step = cols.step;
         sc.f32 = 1;
