@@ -522,8 +522,8 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // stopped at this step (set by its SpMV launch) or earlier; at a happy
     // breakdown at this step y~_{j-1}, still in Y, is sketched in the place of w_j
-    // (which need not be finite: the products of the step may have overflowed); a
-    // dense sketch, applied to the slot of w_j after this launch, finds it there
+    // (which need not be finite: the products of the step may have overflowed), from
+    // the slot of w_j, where a dense sketch, applied after this launch, finds it too
     const bool stop_here = c.iscal[0] == 1 && c.iscal[3] == j && j >= 1;
     if (c.iscal[0] && c.iscal[3] <= j && (!stop_here || c.identity)) return;
     const int G = gridDim.x;
@@ -590,10 +590,10 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
     unsigned long long nkey = 0;
     const int64_t r0 = (int64_t)blockIdx.x * c.rows_per_cta;
     const int64_t r1 = min(c.n, r0 + c.rows_per_cta);
-    if (stop_here && !c.sparse) {
+    if (stop_here) {   // (a thread's own rows of the loop below)
         double *wj = c.V + vcol(c, j);
         for (int64_t r = r0 + threadIdx.x; r < r1; r += kUpdThreads) wj[r] = c.Y[r];
-        return;
+        if (!c.sparse) return;
     }
     double *wn = c.V + vcol(c, j + 1);
     // window offsets newest first: woffr[b] locates w_{j-b}
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(kUpdThreads, KW <= 2 ? 2 : 1) k_arnoldi_update
             if (xr < rn) {
                 const int64_t r = r0 + xr;
                 const double y = cur.y[u];
-                const double wjr = stop_here ? y : cur.w[u][0];
+                const double wjr = cur.w[u][0];
                 if (do_update) {
                     double w = sigma * y;
 #pragma unroll
