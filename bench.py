@@ -37,11 +37,11 @@ HBM_PEAK_FALLBACK = 6800.0
 # DRAM bytes (read + write) per Arnoldi step, summed over the spmv and update
 # kernels of one ncu capture of those kernels as they stand; keyed by workload,
 # basis dtype and sketch, and removed whenever those kernels change.
-FP32_STEP_TRAFFIC = 1059.0e6   # DRAM bytes per FP32 step at N = 16.8M (ncu, the current kernels)
+FP32_STEP_TRAFFIC = 1054.7e6   # DRAM bytes per FP32 step at N = 16.8M (ncu, the current kernels)
 # ncu dram bytes per Arnoldi step, for step kernels unchanged since their capture;
 # k_arnoldi_persist is one launch for all m steps: per-step bytes are the
 # difference of two captures (m = 40 and m = 12) over 28 steps; the FP32 entry
-# is the two step kernels of one step (spmv 669.1 MB + update 389.9 MB)
+# is the two step kernels of one step (spmv 668.2 MB + update 386.5 MB)
 NCU_TRAFFIC_PER_STEP = {("cd3d_n100", "f64", "sparse_sign", True): 8.3e6,
                         ("cd3d_n100", "f64", "sparse_sign", False): None,
                         ("cd3d_n256_fp32", "f32", "sparse_sign", False): FP32_STEP_TRAFFIC}

@@ -7,7 +7,8 @@
 // and of its coefficients, which H and the relation for S A v_j then use.
 //
 // The whole recurrence (all m steps) runs in one cooperative launch of one
-// CTA per SM.  CTA g owns R consecutive rows (whole SELL-32 slices) and keeps
+// CTA per SM at most (of a small problem two launches fit side by side, see
+// kShortRows).  CTA g owns R consecutive rows (whole SELL-32 slices) and keeps
 // its rows of the k window vectors w_{j-k+1} .. w_j and of y~ = A w_j in
 // shared memory for the whole process.  Per step HBM therefore sees the
 // operator, the gathered entries of w_j and the store of w_{j+1}: the window
@@ -34,10 +35,10 @@
 // roundoff of ||A v_j||).  The last column (and the column at a happy
 // breakdown, where no further vector is formed) is sketched directly.
 //
-// Cross-CTA sums: exact integer sums of the dots and sketch partials, added
-// with 64-bit global atomics (the order does not matter; see push_sums).  Every barrier wait is bounded by a clock64
-// budget: past it the kernel records SKF_ERR_TIMEOUT, and every CTA returns
-// at its next barrier.
+// Cross-CTA sums: integer sums of the dots and sketch partials, added with
+// 64-bit global atomics (the order does not matter; see flush_sums).  Every
+// barrier wait is bounded by a clock64 budget: past it the kernel records
+// SKF_ERR_TIMEOUT, and every CTA returns at its next barrier.
 #include <math.h>
 
 #include <algorithm>

@@ -1650,7 +1650,7 @@ __global__ void __launch_bounds__(kThreads) k_levels(TailMethods tm, int lev0, i
 
 // y = R^{-1} q_acc, z = vscale .* y: one warp (warp_back_solve);
 // ILL_CONDITIONED when R has a zero pivot or the estimate of cond(R)
-// (k_tri_right) exceeds cond_max.
+// (cond_estimate) exceeds cond_max.
 template <int K>
 __global__ void __launch_bounds__(32) k_coeffs(TailMethods tm) {
     const TailCtx &c = tm.c[blockIdx.x];

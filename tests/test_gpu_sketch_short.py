@@ -25,3 +25,16 @@ def test_short_columns(skf, N, noalloc):
         assert not got[:, 1].any()
         for c in (0, 2):
             assert np.linalg.norm(got[:, c] - want[:, c]) <= 1e-14 * np.linalg.norm(want[:, c])
+
+
+# stripes of 64 / 65 rows (8 / 4 copies of the bins by lane) and of 128 / 129 (4 / the
+# general pattern, one)
+@pytest.mark.parametrize("s", [512, 520, 1024, 1032])
+def test_bin_copies_at_the_stripe_widths(skf, s):
+    N = 20_011
+    X = np.random.default_rng(s).standard_normal((N, 3))
+    S = skf.Sketch(skf.SPARSE_SIGN, N, s, 8, 21)
+    got = skf.sketch_apply(S, torch.as_tensor(X, device="cuda")).cpu().numpy()
+    want = OSketch("sparse_sign", N, s, 8, 21) @ X
+    for c in range(3):
+        assert np.linalg.norm(got[:, c] - want[:, c]) <= 1e-14 * np.linalg.norm(want[:, c])
