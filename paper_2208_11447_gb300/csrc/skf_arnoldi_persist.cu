@@ -1355,7 +1355,7 @@ int64_t persist_max_rows_f64() {
         return 0;
     }
     int R = 32;
-    while (persist_smem(R + 32, 2, 16 * 64, true) + 4096 <= (size_t)optin) R += 32;
+    while (persist_smem(R + 32, 1, 16 * 64, true) + 4096 <= (size_t)optin) R += 32;
     return (int64_t)R * num_sms();
 }
 

@@ -498,7 +498,8 @@ inline double solve_seconds(int m, double n, double nnz, int value_bytes, int ba
 
 constexpr int kPersistLevels = 3;
 void persist_partition(int64_t n, int level, int *G, int64_t *rows);
-// rows up to which the persistent form holds an FP64 basis (k = 2, a sketch of few rows)
+// rows up to which the persistent form holds an FP64 basis (k = 1, a sketch of few
+// rows: 3.8e6; k = 2: 1.9e6)
 int64_t persist_max_rows_f64();
 
 // Fixed-point sketch accumulation.  A value x is rounded to the integer

@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 def test_no_copy_that_nothing_reads(skf):
-    A = convdiff_2d(1500, (60.0, 50.0))
+    A = convdiff_2d(2000, (60.0, 50.0))
     csr = [torch.as_tensor(v, device="cuda") for v in (A.rowptr, A.colind, A.values)]
     first = skf.upload_csr(*csr)   # (one-time allocations)
     torch.cuda.synchronize()
